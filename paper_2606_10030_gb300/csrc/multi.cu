@@ -31,6 +31,7 @@ constexpr int kMultiThreads = 512;
 constexpr int kMultiProbe = 128;
 constexpr unsigned long long kEmpty64 = ~0ull;
 constexpr int kMultiFull = 1;  // status: a key found no slot
+constexpr int kMultiBufs = 7;  // uint32 arrays of the finalisation, one element a slot
 
 // SplitMix64's output function (Steele, Lea and Flood 2014), a bijective mixer.
 __device__ __forceinline__ uint64_t mix64(uint64_t z) {
@@ -358,7 +359,7 @@ static agg_status multi_run(MultiArgs a, int64_t S, cudaStream_t s, agg_multi** 
   const size_t status_off = bytes;
   bytes += 256;
   const size_t fin_off = bytes;
-  bytes += 6 * k4 + radix_tmp_bytes(S1) + 256;
+  bytes += kMultiBufs * k4 + radix_tmp_bytes(S1) + 256;
   char* mem = nullptr;
   AGG_CUDA_TRY(dev_malloc_async((void**)&mem, bytes, s));
   struct Free {
@@ -401,10 +402,10 @@ static agg_status multi_run(MultiArgs a, int64_t S, cudaStream_t s, agg_multi** 
   // finalise: compact the occupied slots, order them by (high word, low word)
   // with two stable radix sorts of (word, compact index) pairs, gather
   PhaseTimer pt(AGG_PHASE_FINALIZE, s);
-  uint32_t* buf[7];
-  for (int k = 0; k < 7; ++k) buf[k] = (uint32_t*)(mem + fin_off + (size_t)k * k4);
+  uint32_t* buf[kMultiBufs];
+  for (int k = 0; k < kMultiBufs; ++k) buf[k] = (uint32_t*)(mem + fin_off + (size_t)k * k4);
   uint32_t *klo = buf[0], *khi = buf[1], *slot = buf[2], *idx = buf[3];
-  void* rtmp = (void*)(((uintptr_t)(mem + fin_off + 7 * k4) + 255) & ~(uintptr_t)255);
+  void* rtmp = (void*)(((uintptr_t)(mem + fin_off + kMultiBufs * k4) + 255) & ~(uintptr_t)255);
   const int64_t* dd = (const int64_t*)dcount;
   const int g = (int)std::max<int64_t>(1, std::min<int64_t>((S1 + 255) / 256, (int64_t)di.sm_count * 8));
   multi_compact<<<g, 256, 0, s>>>(a.keys, a.cnt, S1, a.mask, klo, khi, slot, dcount);

@@ -128,6 +128,20 @@ def test_multi_matches_the_single_key_group_by():
         assert np.array_equal(res["cols"][0][f], r[f])
 
 
+def test_multi_two_million_groups():
+    """A table of millions of slots: its finalisation arrays and radix scratch fill one block to the end."""
+    n = 3_000_001
+    lo = dg.keys_uniform(n, 3_000_000, 11)
+    v = dg.values("i64", n, 12)
+    res = run(lo, None, [v], [agg.AGG_ALL], None)
+    order = np.argsort(lo, kind="stable")
+    keys, first = np.unique(lo[order], return_index=True)
+    assert np.array_equal(res["keys"], keys.astype(np.uint64))
+    assert np.array_equal(res["count"], np.diff(np.append(first, n)))
+    for name, f in (("sum", np.add), ("min", np.minimum), ("max", np.maximum)):
+        assert np.array_equal(res["cols"][0][name], f.reduceat(v[order], first))
+
+
 def test_multi_2p26_rows_two_keys_three_columns_filtered():
     """2^26 rows: low key over 4096 keys, high key over 16 values, int64 / float32 /
     float64 columns, a filter that keeps about half the rows."""
