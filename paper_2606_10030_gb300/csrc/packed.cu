@@ -68,7 +68,7 @@ __global__ void __launch_bounds__(kBlock) packed_scan(const PackDesc* __restrict
   }
   Partial p;
   a.to_partial(p, 0);
-  p = block_reduce<kBlock>(p);
+  p = block_reduce<Traits<DT>::FP, kBlock>(p);
   if (threadIdx.x == 0) parts[part_base + blockIdx.x] = p;
 }
 

@@ -17,18 +17,18 @@
 //   float64   a 128-bit fixed-point integer at the scale of the largest
 //             exponent seen (integer operations only: GB300 issues few
 //             float64 operations), uint64 images for min/max.
-// Block partials carry the sum as a float64 pair (hi, lo); the final merge is
-// a float64 double-double sum in a fixed order, so the result is
-// deterministic for a given grid.
+// Float sums leave the threads as 128-bit fixed-point numbers (Fix128), and
+// warps, blocks and the grid merge them with integer additions; one thread
+// converts the total to float64 at the end. The order is fixed, so the result
+// is deterministic for a given grid. Measured against float64 TwoSum merges in
+// every shuffle step: 2^20 int32 rows 17.7 -> 8.7 us a call, 10^8 float64
+// rows 207 -> 178 us (with the scale started from the warp's first rows).
 //
-// Error bound of a float SUM. Every partial also carries eb, a bound on
-// |hi + lo - (exact sum of its rows)|, built from the roundings that can
-// occur: per thread, those of the compensation word of a float32 pair (each
-// at most 2^-24 of the word's new value, tracked as the word's largest
-// magnitude) or the truncations of the float64 fixed-point sum (less than one
-// unit each, at most two per row); per merge, the two float64 roundings of
-// the low words. The result's err_bound adds the final rounding of hi + lo
-// and the oracle's own rounding of the exact sum, so that
+// Error bound of a float SUM. It adds up the roundings that can occur: per
+// thread, those of the compensation word of a float32 pair (each at most 2^-24
+// of the word's new value, tracked as the word's largest magnitude); the
+// fixed-point units lost (less than one per add, rescale or merge); the final
+// rounding of hi + lo and the oracle's own rounding of the exact sum, so that
 // |sum_f - (exact sum rounded to float64)| <= err_bound.
 #include <map>
 #include <mutex>
@@ -39,8 +39,10 @@ namespace agg {
 
 // The scan. Rows [0, head) and the ragged tail are folded with scalar loads by
 // the first threads of the grid; the 16-byte-aligned body with vector loads.
+// Six blocks a SM (40 registers) keep 98 KB of loads in flight a SM; int64
+// MIN/MAX needs 54 registers and runs four.
 template <int DT, bool SUM, bool MM>
-__global__ void __launch_bounds__(kBlock) reduce_scan(const typename Traits<DT>::T* __restrict__ col,
+__global__ void __launch_bounds__(kBlock, DT == AGG_I64 && MM ? 4 : 6) reduce_scan(const typename Traits<DT>::T* __restrict__ col,
                                                       int64_t n, int64_t head, Partial* __restrict__ parts,
                                                       int part_base, unsigned* ticket, agg_scalar* out,
                                                       uint32_t ops, int64_t count_total, int finalize) {
@@ -57,6 +59,14 @@ __global__ void __launch_bounds__(kBlock) reduce_scan(const typename Traits<DT>:
     if (g < n - tail0) { a.fold(col[tail0 + g]); ++rows; }
     const uint4* v = reinterpret_cast<const uint4*>(col + head);
     const int64_t stride = (int64_t)gridDim.x * kBlock * kUnroll;
+    if constexpr (DT == AGG_F64 && SUM) {
+      // start the fixed-point sum one binade above the largest of the warp's
+      // first 64 rows: a thread that raises its own scale row by row sends the
+      // warp through the slow path some hundred times
+      const int64_t i0 = (int64_t)blockIdx.x * kBlock * kUnroll + threadIdx.x;
+      const uint4 r = i0 < nv ? ld_stream_v4(v + i0) : make_uint4(0, 0, 0, 0);
+      a.fx.start(__reduce_max_sync(0xffffffffu, max((r.y >> 20) & 0x7FFu, (r.w >> 20) & 0x7FFu)));
+    }
     for (int64_t base = (int64_t)blockIdx.x * kBlock * kUnroll + threadIdx.x; base < nv; base += stride) {
       uint4 r[kUnroll];
 #pragma unroll
@@ -75,7 +85,7 @@ __global__ void __launch_bounds__(kBlock) reduce_scan(const typename Traits<DT>:
   }
   Partial p;
   a.to_partial(p, rows);
-  p = block_reduce<kBlock>(p);
+  p = block_reduce<Traits<DT>::FP, kBlock>(p);
   __shared__ int s_last;
   if (threadIdx.x == 0) {
     parts[part_base + blockIdx.x] = p;

@@ -12,12 +12,22 @@
 
 namespace agg {
 
-struct Partial {  // one block's partial aggregate
-  int64_t si;     // integer sum
-  double hi, lo;  // float sum, unevaluated hi + lo
-  uint64_t mn, mx;  // order-preserving images of min / max
-  double eb;      // bound on |hi + lo - exact sum of the rows| (float columns)
+// One block's partial aggregate (48 bytes). Integer columns use w0 (the sum mod
+// 2^64); float columns hold their sum as the 128-bit fixed-point number w1:w0
+// of Fix128 at the scale of exponent E, so that warps, blocks and the grid
+// merge with integer additions: GB300 issues few float64 operations, and a
+// float64 TwoSum in every shuffle step made a 2^20-row int32 scan 17 us long
+// and put 40 us on every float64 scan.
+struct Partial {
+  uint64_t w0, w1;
+  uint64_t mn, mx;   // order-preserving images of min / max
+  int32_t E;         // exponent field the fixed-point sum is scaled to (0: no value yet)
+  uint32_t special;  // float: kPosInf | kNegInf | kNan seen
+  float eb;          // float32: bound on the roundings of the threads' compensation words
+  uint32_t pad;
 };
+static_assert(sizeof(Partial) == 48, "partials of the static scratch");
+constexpr uint32_t kPosInf = 1, kNegInf = 2, kNan = 4;
 
 template <int DT> struct Traits;
 template <> struct Traits<AGG_I32> { using T = int32_t; static constexpr bool FP = false; };
@@ -56,12 +66,10 @@ struct Acc<DT, SUM, MM, false> {
     }
   }
   __device__ void to_partial(Partial& p, uint32_t) const {
-    p.si = s;
-    p.hi = 0.0;
-    p.lo = 0.0;
+    p = Partial{};
+    p.w0 = (uint64_t)s;
     p.mn = img_i64((int64_t)mn);
     p.mx = img_i64((int64_t)mx);
-    p.eb = 0.0;
   }
 };
 
@@ -69,16 +77,12 @@ template <class F> struct FpImg;
 template <> struct FpImg<float> {
   using U = uint32_t;
   __device__ static U img(float x) { return img_f32(x); }
-  __device__ static uint64_t widen(U m) {  // f32 image -> image of the same value as f64
-    if (m == 0xFFFFFFFFu) return ~0ull;    // identity of min
-    if (m == 0u) return 0ull;              // identity of max
-    return img_f64((double)f32_of_img(m));
-  }
+  __device__ static double value(uint64_t m) { return (double)f32_of_img((uint32_t)m); }
 };
 template <> struct FpImg<double> {
   using U = uint64_t;
   __device__ static U img(double x) { return img_f64(x); }
-  __device__ static uint64_t widen(U m) { return m; }
+  __device__ static double value(uint64_t m) { return f64_of_img(m); }
 };
 
 // float64 SUM on the integer pipes: a 128-bit two's-complement fixed-point
@@ -90,9 +94,8 @@ template <> struct FpImg<double> {
 // 2^(E - 1075 - kFixGuard), 2^-83 of the largest row); a row with a larger
 // exponent shifts the sum right (again less than a unit lost). Sums of up to
 // 2^43 rows per thread cannot overflow (|m x 2^kFixGuard| < 2^84). A guard of
-// 31 bits keeps the fast path's shift below one word. Infinities and NaNs are added in
-// float64 on the side, so that a column holding one sums to a non-finite
-// value (which one is unspecified, as for the other float paths).
+// 31 bits keeps the fast path's shift below one word. Infinities and NaNs are noted
+// on the side, so that a column holding one sums to a non-finite value.
 // GB300 issues few float64 operations per clock (a TwoSum per row held the
 // float64 scan to 0.6 TB/s); this takes only integer operations per row.
 constexpr int kFixGuard = 31;
@@ -102,14 +105,18 @@ struct Fix128 {
   uint32_t nneg;  // negative rows added on the fast path as ~v, each still owing +1
   int E;
   int base;       // E - kFixGuard: a row of exponent field e sits e - base bits up
-  double special;
+  uint32_t special;  // kPosInf | kNegInf | kNan
   __device__ void init() {
     lo = 0;
     hi = 0;
     nneg = 0;
     E = 0;
     base = -kFixGuard;
-    special = 0.0;
+    special = 0;
+  }
+  // Scale for rows of exponent fields up to ef + 1 (the sum so far is zero or exact).
+  __device__ __forceinline__ void start(uint32_t ef) {
+    if (ef > 0 && ef < 0x7FEu && (int)ef >= E) rescale((int)ef + 1);
   }
   // -v = ~v + 1: the fast path adds ~v and counts the +1s, added here.
   __device__ __forceinline__ void fold_neg() {
@@ -117,19 +124,22 @@ struct Fix128 {
     hi += lo < nneg ? 1ull : 0ull;
     nneg = 0;
   }
+  // (vhi:vlo) >> k for k >= 1, rounding toward minus infinity (less than one unit).
+  __device__ static __forceinline__ void shift_right(uint64_t& vlo, uint64_t& vhi, int k) {
+    if (k >= 127) {
+      vlo = (int64_t)vhi < 0 ? ~0ull : 0ull;
+      vhi = vlo;
+    } else if (k >= 64) {
+      vlo = (uint64_t)((int64_t)vhi >> (k - 64));
+      vhi = (uint64_t)((int64_t)vhi >> 63);
+    } else {
+      vlo = (vlo >> k) | (vhi << (64 - k));
+      vhi = (uint64_t)((int64_t)vhi >> k);
+    }
+  }
   __device__ __forceinline__ void rescale(int e) {  // e > E
     fold_neg();
-    const int k = e - E;
-    if (k >= 127) {
-      lo = (int64_t)hi < 0 ? ~0ull : 0ull;
-      hi = lo;
-    } else if (k >= 64) {
-      lo = (uint64_t)((int64_t)hi >> (k - 64));
-      hi = (uint64_t)((int64_t)hi >> 63);
-    } else {
-      lo = (lo >> k) | (hi << (64 - k));
-      hi = (uint64_t)((int64_t)hi >> k);
-    }
+    shift_right(lo, hi, e - E);
     E = e;
     base = e - kFixGuard;
   }
@@ -165,7 +175,7 @@ struct Fix128 {
     }
     fold_neg();
     if (ef == 0x7FF) {  // infinity or NaN
-      special += __longlong_as_double((long long)u);
+      special |= (u & 0x000FFFFFFFFFFFFFull) ? kNan : (int64_t)u < 0 ? kNegInf : kPosInf;
       return;
     }
     const int e = ef > 0 ? ef : 1;  // subnormals: exponent 1, no implicit bit
@@ -189,33 +199,32 @@ struct Fix128 {
     lo += vlo;
     hi += vhi + (lo < vlo ? 1ull : 0ull);
   }
-  // The sum as an unevaluated float64 pair (rel. error about 2^-106 before
-  // scaling): the 128-bit integer in three chunks that float64 holds exactly,
-  // added with TwoSum, then scaled by 2^(E - 1075 - kFixGuard).
-  __device__ void to_pair(double& h, double& l) const {
-    const uint64_t m43 = (1ull << 43) - 1ull;
-    const double q0 = (double)(lo & m43);
-    const double q1 = (double)(((lo >> 43) | (hi << 21)) & m43);
-    const double q2 = (double)((int64_t)hi >> 22);
-    double s1, e1, s2, e2;
-    two_sum(ldexp(q2, 86), ldexp(q1, 43), s1, e1);
-    two_sum(s1, q0, s2, e2);
-    double t, f;
-    two_sum(s2, e1 + e2, t, f);
-    const int sc = E - 1075 - kFixGuard;
-    h = ldexp(t, sc) + special;
-    l = special == 0.0 ? ldexp(f, sc) : 0.0;
-  }
-  // Bound on |h + l - exact sum| after `rows` adds: each add loses less than
-  // one unit 2^(E - 1075 - kFixGuard) (a row far below E), each rescale less
-  // than one unit of the new scale; to_pair rounds e1 + e2 (under 2^-104 of
-  // the sum) and may round h and l into the subnormal range.
-  __device__ double error_bound(uint32_t rows, double h, double l) const {
-    if (special != 0.0) return __longlong_as_double(0x7ff0000000000000ll);
-    if (E == 0) return 0.0;
-    return ldexp(2.0 * (double)rows, E - 1075 - kFixGuard) + (fabs(h) + fabs(l)) * 0x1p-100 + 0x1p-1072;
-  }
 };
+
+// The sum of a partial as an unevaluated float64 pair (rel. error about 2^-106
+// before scaling): the 128-bit integer in three chunks that float64 holds
+// exactly, added with TwoSum, then scaled by 2^(E - 1075 - kFixGuard).
+__device__ inline void fix_to_pair(const Partial& p, double& h, double& l) {
+  const uint64_t lo = p.w0, hi = p.w1;
+  const uint64_t m43 = (1ull << 43) - 1ull;
+  const double q0 = (double)(lo & m43);
+  const double q1 = (double)(((lo >> 43) | (hi << 21)) & m43);
+  const double q2 = (double)((int64_t)hi >> 22);
+  double s1, e1, s2, e2;
+  two_sum(q2 * 0x1p86, q1 * 0x1p43, s1, e1);
+  two_sum(s1, q0, s2, e2);
+  double t, f;
+  two_sum(s2, e1 + e2, t, f);
+  const int sc = p.E - 1075 - kFixGuard;
+  h = ldexp(t, sc);
+  l = ldexp(f, sc);
+  if (p.special) {  // both infinities, or a NaN: NaN
+    l = 0.0;
+    h = __longlong_as_double(p.special == kPosInf   ? 0x7ff0000000000000ll
+                             : p.special == kNegInf ? (long long)0xfff0000000000000ull
+                                                    : 0x7ff8000000000000ll);
+  }
+}
 
 template <int DT, bool SUM, bool MM>
 struct Acc<DT, SUM, MM, true> {
@@ -273,69 +282,90 @@ struct Acc<DT, SUM, MM, true> {
   }
   // rows: the number of values this thread folded.
   __device__ void to_partial(Partial& p, uint32_t rows) const {
-    p.si = 0;
-    p.eb = 0.0;
-    if (F64 && SUM) {
+    p = Partial{};
+    if (SUM) {
       Fix128 f = fx;
-      f.fold_neg();
-      f.to_pair(p.hi, p.lo);
-      p.eb = f.error_bound(rows, p.hi, p.lo);
-    } else {
-      p.hi = (double)s;
-      p.lo = (double)c;
-      // TwoSum leaves s + c short only by the roundings of c: each at most
-      // 2^-24 of |c| after the add (2^-150 when c is subnormal)
-      if (SUM && !F64) {
-        p.eb = (isfinite(p.hi) && isfinite(p.lo))
-                   ? (double)rows * ((double)cmax * (0x1p-24 * (1.0 + 0x1p-23)) + 0x1p-150)
-                   : __longlong_as_double(0x7ff0000000000000ll);
+      if (!F64) {
+        // the float32 pair as two rows of a fixed-point sum (s's exponent and
+        // 31 binades below it: all of c's bits but a guard's worth)
+        f.init();
+        f.add((uint64_t)__double_as_longlong((double)s));
+        f.add((uint64_t)__double_as_longlong((double)c));
+        // TwoSum leaves s + c short only by the roundings of c: each at most
+        // 2^-24 of |c| after the add (2^-150 when c is subnormal)
+        p.eb = __fmul_ru(__uint2float_ru(rows), __fadd_ru(__fmul_ru((float)cmax, 0x1.000002p-24f), 0x1p-149f));
       }
+      f.fold_neg();
+      p.w0 = f.lo;
+      p.w1 = f.hi;
+      p.E = f.E;
+      p.special = f.special;
     }
-    p.mn = FpImg<T>::widen(mn);
-    p.mx = FpImg<T>::widen(mx);
+    p.mn = mn == (U)~(U)0 ? ~0ull : (uint64_t)mn;
+    p.mx = mx;
   }
 };
 
 // ---------------------------------------------------------------------------
 // Warp / block reduction of Partial values (fixed shuffle tree).
 // ---------------------------------------------------------------------------
+template <bool FP>
 __device__ __forceinline__ void combine(Partial& a, const Partial& b) {
-  a.si += b.si;
-  double s, e;
-  two_sum(a.hi, b.hi, s, e);
-  a.hi = s;
-  const double r1 = e + b.lo;  // rounded: at most 2^-53 |r1| (+ 2^-1075)
-  a.lo += r1;                  // rounded: at most 2^-53 |a.lo| (+ 2^-1075)
-  a.eb = a.eb + b.eb + (fabs(r1) + fabs(a.lo)) * 0x1p-53 + 0x1p-1074;
+  if (FP) {
+    // the sum of the smaller exponent is shifted to the other's scale (less
+    // than one unit lost), then added
+    uint64_t blo = b.w0, bhi = b.w1;
+    if (b.E > a.E) {
+      Fix128::shift_right(a.w0, a.w1, b.E - a.E);
+      a.E = b.E;
+    } else if (b.E < a.E) {
+      Fix128::shift_right(blo, bhi, a.E - b.E);
+    }
+    a.w0 += blo;
+    a.w1 += bhi + (a.w0 < blo ? 1ull : 0ull);
+    a.special |= b.special;
+    a.eb = __fadd_ru(a.eb, b.eb);
+  } else {
+    a.w0 += b.w0;
+  }
   a.mn = min(a.mn, b.mn);
   a.mx = max(a.mx, b.mx);
 }
 
+__device__ __forceinline__ Partial empty_partial() {
+  Partial p{};
+  p.mn = ~0ull;
+  return p;
+}
+
+template <bool FP>
 __device__ __forceinline__ Partial shfl_xor(const Partial& p, int m) {
-  Partial q;
-  q.si = __shfl_xor_sync(0xffffffffu, p.si, m);
-  q.hi = __shfl_xor_sync(0xffffffffu, p.hi, m);
-  q.lo = __shfl_xor_sync(0xffffffffu, p.lo, m);
+  Partial q{};
+  q.w0 = __shfl_xor_sync(0xffffffffu, p.w0, m);
+  if (FP) {
+    q.w1 = __shfl_xor_sync(0xffffffffu, p.w1, m);
+    q.E = __shfl_xor_sync(0xffffffffu, p.E, m);
+    q.special = __shfl_xor_sync(0xffffffffu, p.special, m);
+    q.eb = __shfl_xor_sync(0xffffffffu, p.eb, m);
+  }
   q.mn = __shfl_xor_sync(0xffffffffu, p.mn, m);
   q.mx = __shfl_xor_sync(0xffffffffu, p.mx, m);
-  q.eb = __shfl_xor_sync(0xffffffffu, p.eb, m);
   return q;
 }
 
 // Block-wide reduction; the result is valid in thread 0.
-template <int BLOCK>
+template <bool FP, int BLOCK>
 __device__ Partial block_reduce(Partial p) {
   __shared__ Partial sm[BLOCK / 32];
 #pragma unroll
-  for (int m = 16; m >= 1; m >>= 1) combine(p, shfl_xor(p, m));
+  for (int m = 16; m >= 1; m >>= 1) combine<FP>(p, shfl_xor<FP>(p, m));
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
   if (l == 0) sm[w] = p;
   __syncthreads();
   if (w == 0) {
-    if (l < BLOCK / 32) p = sm[l];
-    else p = Partial{0, 0.0, 0.0, ~0ull, 0ull, 0.0};
+    p = l < BLOCK / 32 ? sm[l] : empty_partial();
 #pragma unroll
-    for (int m = 16; m >= 1; m >>= 1) combine(p, shfl_xor(p, m));
+    for (int m = BLOCK / 64; m >= 1; m >>= 1) combine<FP>(p, shfl_xor<FP>(p, m));
   }
   return p;
 }
@@ -345,19 +375,20 @@ __device__ Partial block_reduce(Partial p) {
 template <int DT, int BLOCK>
 __device__ void merge_partials(const Partial* parts, int np, agg_scalar* out, uint32_t ops,
                                int64_t count) {
-  Partial acc{0, 0.0, 0.0, ~0ull, 0ull, 0.0};
+  constexpr bool FP = Traits<DT>::FP;
+  Partial acc = empty_partial();
   for (int i = threadIdx.x; i < np; i += BLOCK) {
-    Partial q;
-    q.si = __ldcg(&parts[i].si);
-    q.hi = __ldcg(&parts[i].hi);
-    q.lo = __ldcg(&parts[i].lo);
-    q.mn = __ldcg(&parts[i].mn);
-    q.mx = __ldcg(&parts[i].mx);
-    q.eb = __ldcg(&parts[i].eb);
-    combine(acc, q);
+    const uint4* q4 = reinterpret_cast<const uint4*>(&parts[i]);
+    union {
+      uint4 v[3];
+      Partial p;
+    } q;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) q.v[k] = __ldcg(q4 + k);
+    combine<FP>(acc, q.p);
   }
   __syncthreads();
-  acc = block_reduce<BLOCK>(acc);
+  acc = block_reduce<FP, BLOCK>(acc);
   if (threadIdx.x != 0) return;
   agg_scalar r;
   r.count = count;
@@ -365,27 +396,37 @@ __device__ void merge_partials(const Partial* parts, int np, agg_scalar* out, ui
   r.ops = ops;
   r.err_bound = 0.0;
   const double nan = __longlong_as_double(0x7ff8000000000000ll);
-  if (Traits<DT>::FP) {
-    double s = acc.hi + acc.lo;
+  if constexpr (FP) {
+    const double inf = __longlong_as_double(0x7ff0000000000000ll);
+    double hi, lo;
+    fix_to_pair(acc, hi, lo);
+    double s = hi + lo;
     r.sum_i = 0;
     r.sum_f = s;
-    // the partials' bound, plus the rounding of hi + lo and the oracle's own
-    // rounding of the exact sum (each at most 2^-53 of the value), plus a
-    // margin for the roundings of the bound's own sums
+    // Bound on |s - exact sum|: the threads' compensation words (float32); the
+    // fixed-point units lost, less than one per add, per rescale and per merge
+    // of a thread's sum (float64: at most three a row; float32: a thread that
+    // folded a row adds two words, so at most five a row); fix_to_pair (under
+    // 2^-104 of the sum, and the subnormal range); the rounding of hi + lo and
+    // the oracle's own rounding of the exact sum (each at most 2^-53 of the
+    // value); and a margin for the roundings of the bound's own sums.
     if (ops & (AGG_SUM | AGG_AVG)) {
-      r.err_bound = (acc.eb + fabs(s) * 0x1p-52 + 0x1p-1073) * (1.0 + 0x1p-40);
+      const double units = acc.E ? ldexp((sizeof(typename Traits<DT>::T) == 8 ? 3.0 : 5.0) * (double)count,
+                                         acc.E - 1075 - kFixGuard)
+                                 : 0.0;
+      r.err_bound = ((double)acc.eb + units + fabs(s) * (0x1p-52 + 0x1p-99) + 0x1p-1072) * (1.0 + 0x1p-40);
       // a column holding an infinity or a NaN has no finite bound
-      if (!isfinite(s) || !isfinite(r.err_bound)) r.err_bound = __longlong_as_double(0x7ff0000000000000ll);
+      if (acc.special || !isfinite(s) || !isfinite(r.err_bound)) r.err_bound = inf;
     }
     r.avg = count ? s / (double)count : nan;
-    r.min_f = count ? f64_of_img(acc.mn) : __longlong_as_double(0x7ff0000000000000ll);
-    r.max_f = count ? f64_of_img(acc.mx) : __longlong_as_double((long long)0xfff0000000000000ull);
+    r.min_f = count ? FpImg<typename Traits<DT>::T>::value(acc.mn) : inf;
+    r.max_f = count ? FpImg<typename Traits<DT>::T>::value(acc.mx) : -inf;
     r.min_i = 0;
     r.max_i = 0;
   } else {
-    r.sum_i = acc.si;
-    r.sum_f = (double)acc.si;
-    r.avg = count ? (double)acc.si / (double)count : nan;
+    r.sum_i = (int64_t)acc.w0;
+    r.sum_f = (double)r.sum_i;
+    r.avg = count ? r.sum_f / (double)count : nan;
     r.min_i = count ? i64_of_img(acc.mn) : LLONG_MAX;
     r.max_i = count ? i64_of_img(acc.mx) : LLONG_MIN;
     r.min_f = 0.0;
