@@ -194,12 +194,11 @@ typedef struct agg_options {
   int32_t strategy;        /* agg_strategy */
   int32_t block_threads;   /* threads per block of the build kernel; 0 = default */
   int32_t blocks_per_sm;   /* resident blocks per SM; 0 = occupancy limit */
-  int32_t smem_slots;      /* shared-memory table slots (power of two, <= 8192); 0 = from the sketch */
+  int32_t smem_slots;      /* shared-memory table slots (power of two, <= 8192; a build uses at most 4096, 2048 for
+                              partitioned MIN/MAX builds and float64 MIN/MAX); 0 = from the sketch */
   int64_t table_slots;     /* global table slots (power of two); 0 = from the sketch */
   uint64_t sample_offset;  /* offset of the strided key sample (pass a seeded draw) */
-  int32_t items_per_thread;/* rows a thread folds per iteration of the build's vector loop: 4 or 8; 0 = 8
-                              for the unpartitioned shared-memory build of an integer column without
-                              frequent keys, else 4 */
+  int32_t items_per_thread;/* rows a thread folds per iteration of the build's vector loop: 4 or 8; 0 = 4 */
   int32_t partition;       /* hash-partition the rows before a hash build: 0 = automatic (when the
                               shared tables would spill or the global table exceeds half of L2; two
                               levels above ~600k distinct keys), 1 = one level (256 partitions),
@@ -433,11 +432,12 @@ agg_status agg_distinct_estimate(const uint32_t* keys_dev, int64_t n, double* es
  * query's strategy (query.strategy: AUTO = the rule, LEARNED = the installed
  * network, or SMEM / GLOBAL) and table sizes, and allocates everything; one
  * host synchronisation. In a batch every query runs a hash strategy: a query
- * for which SORT is chosen runs on shared-memory tables (identical results).
+ * for which SORT is chosen runs on shared-memory tables, or on its global table
+ * when the sample is flat over far more keys (identical results).
  * agg_batch_run performs the device work (tables cleared, one persistent
- * build kernel over (query, tile) work items, 64 Ki rows unless agg_batch_tune
- * chose another size, pulled from a device
- * counter, batched finalisation into ascending key order) as a CUDA graph
+ * build kernel over (query, tile) work items, 64 Ki rows (down to 8 Ki for a
+ * batch of few rows) unless agg_batch_tune chose another size, pulled from a
+ * device counter, batched finalisation into ascending key order) as a CUDA graph
  * captured on the first run and replayed afterwards, then reads back the group
  * counts; synchronous. A table that overflows is regrown (new graph) and the
  * run repeated. Inputs must stay valid and unchanged while the plan is used;

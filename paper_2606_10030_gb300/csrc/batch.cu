@@ -9,7 +9,7 @@
 //
 // Run (device only; captured into a CUDA graph on the first run, replayed
 // after): zero the tables; one persistent build kernel whose blocks pull
-// (query, 64 Ki-row tile) work items from a device counter, so large and small
+// (query, row tile) work items from a device counter, so large and small
 // queries share the GPU without per-query launches; a per-tile shared table
 // is cleared before and merged into the query's global table after each
 // tile. Finalise: queries whose table has at most 4097 slots are each
@@ -20,7 +20,8 @@
 //
 // The sort strategy needs whole-column passes that a tile queue cannot
 // interleave; in a batch, a query for which SORT is chosen runs on
-// shared-memory tables that spill to its global table (identical results).
+// shared-memory tables that spill to its global table, or on the global table
+// alone when the sample is flat over far more keys (identical results).
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -33,8 +34,11 @@
 
 namespace agg {
 
-constexpr int64_t kTileRows = int64_t(1) << 16;  // default rows per work item (agg_batch_tune may change it)
+constexpr int64_t kTileRows = int64_t(1) << 16;  // rows per work item of a large batch (agg_batch_tune may change it)
+constexpr int64_t kMinTileRows = int64_t(1) << 13;
 constexpr int kBatchThreads = 512;
+// Rows a work item of a nominal size holds: a shared table takes at most kEpochRows.
+static int64_t item_rows(int64_t tile_rows) { return std::min(tile_rows, kEpochRows); }
 
 struct BQ {  // one query of a batch, on the device
   const uint32_t* keys;
@@ -47,12 +51,14 @@ struct BQ {  // one query of a batch, on the device
   OutArrays out;
   uint32_t mask;
   int dt, mm, smem, vec;
-  int smem_slots, smem_cap;
+  int smem_slots;
   int gshift;
 };
 
+// Out of line, so that each type's tile gets the kernel's whole register budget
+// (inlined into one kernel, the forty variants spilled a kilobyte a thread).
 template <int DT, bool MM, bool SMEM>
-__device__ void batch_tile(const BQ& q, int64_t r0, int64_t r1, unsigned char* smem) {
+__device__ __noinline__ void batch_tile(const BQ& q, int64_t r0, int64_t r1, unsigned char* smem) {
   BuildArgs a;
   const size_t es = (DT == AGG_I64 || DT == AGG_F64) ? 8 : 4;
   a.keys = q.keys + r0;
@@ -63,21 +69,23 @@ __device__ void batch_tile(const BQ& q, int64_t r0, int64_t r1, unsigned char* s
   a.mask = q.mask;
   a.gshift = q.gshift;
   a.smem_slots = SMEM ? q.smem_slots : 0;
-  a.smem_cap = SMEM ? q.smem_cap : 0;
   a.status = q.status;
   a.progress = nullptr;  // the plan regrows a full table 4x
   a.block_fails = nullptr;
-  STab<DT, MM> st;
+  __shared__ Window s_win;
+  STab<DT, MM, false> t;
   if (SMEM) {
-    st.carve(smem, a.smem_slots);
-    st.clear(a.smem_slots);
+    if (threadIdx.x < 32) s_window<DT>((const typename GV<DT>::T*)a.vals, a.n, &s_win);
+    t.init(smem, a.smem_slots);
+    t.clear();
     __syncthreads();
+    t.set_window(s_win);
   }
-  if (q.vec) build_rows<DT, MM, SMEM, true>(a, st, threadIdx.x, blockDim.x);
-  else build_rows<DT, MM, SMEM, false>(a, st, threadIdx.x, blockDim.x);
+  if (q.vec) build_rows<DT, MM, SMEM, true, true, 1, false>(a, t, 0, blockDim.x);
+  else build_rows<DT, MM, SMEM, false, true, 1, false>(a, t, 0, blockDim.x);
   if (SMEM) {
     __syncthreads();
-    flush_smem<DT, MM>(a, st);
+    s_flush<DT, MM, false, false>(a, t);
   }
 }
 
@@ -92,7 +100,7 @@ __device__ void batch_tile_dt(const BQ& q, int64_t r0, int64_t r1, unsigned char
   }
 }
 
-__global__ void __launch_bounds__(kBatchThreads) batch_build(const BQ* __restrict__ qs, int nq,
+__global__ void __launch_bounds__(kBatchThreads, 2) batch_build(const BQ* __restrict__ qs, int nq,
                                                              const int64_t* __restrict__ tile_prefix,
                                                              int64_t total_tiles, unsigned long long* next_tile,
                                                              int64_t tile_rows) {
@@ -444,7 +452,7 @@ static agg_status plan_alloc(agg_batch_plan* P, cudaStream_t s) {
     b.vals = q.vals;
     b.n = q.n;
     b.tile0 = tile_prefix[i];
-    tile_prefix[i + 1] = tile_prefix[i] + (q.n + P->tile_rows - 1) / P->tile_rows;
+    tile_prefix[i + 1] = tile_prefix[i] + (q.n + item_rows(P->tile_rows) - 1) / item_rows(P->tile_rows);
     b.table = w + qp.table_off;
     b.status = P->status + i;
     b.slot0 = qp.large ? slot_prefix[li++] : -1;
@@ -455,7 +463,6 @@ static agg_status plan_alloc(agg_batch_plan* P, cudaStream_t s) {
     b.smem = qp.strategy == AGG_STRAT_SMEM ? 1 : 0;
     b.vec = (((uintptr_t)q.keys & 15) == 0 && ((uintptr_t)q.vals & 15) == 0) ? 1 : 0;
     b.smem_slots = b.smem ? qp.smem_slots : 0;
-    b.smem_cap = b.smem ? (qp.smem_slots * 3) / 4 : 0;
     char* o = ob + qp.out_off;
     const int64_t cap = qp.cap;
     b.out.keys = (uint32_t*)o;
@@ -471,9 +478,7 @@ static agg_status plan_alloc(agg_batch_plan* P, cudaStream_t s) {
     b.out.avg = (double*)o;
     b.out.d = P->dcount + i;
     if (b.smem) {
-      const bool wide = b.dt == AGG_I64 || b.dt == AGG_F64;
-      const size_t sb = wide ? (b.mm ? stab_bytes<AGG_I64, true>(b.smem_slots) : stab_bytes<AGG_I64, false>(b.smem_slots))
-                             : (b.mm ? stab_bytes<AGG_I32, true>(b.smem_slots) : stab_bytes<AGG_I32, false>(b.smem_slots));
+      const size_t sb = stab_bytes_dt(b.dt, b.mm, false);
       P->build_smem = std::max(P->build_smem, sb);
     }
   }
@@ -509,7 +514,7 @@ static agg_status plan_enqueue(agg_batch_plan* P, cudaStream_t s, int64_t* kerne
   AGG_CUDA_TRY(cudaMemsetAsync(P->work, 0, P->zero_bytes, s));
   if (P->total_tiles > 0) {
     batch_build<<<P->build_grid, kBatchThreads, P->build_smem, s>>>(P->dq, P->nq, P->tile_prefix, P->total_tiles,
-                                                                     P->next_tile, P->tile_rows);
+                                                                     P->next_tile, item_rows(P->tile_rows));
     ++k;
   }
   if (P->nsmall > 0) {
@@ -595,12 +600,24 @@ static void plan_sizes(agg_batch_plan* P, const std::vector<int>& learned) {
     const double est = q.n > 0 ? distinct_estimate(f, &covered) : 1.0;
     const int64_t slots = q.n > 0 ? table_slots_from_sketch(f, q.n) : 1024;
     qp.slots = slots;
-    const int maxs = qp.mm ? 2048 : 4096;
+    const int maxs = stab_max_slots(q.dtype, qp.mm, false);
+    // a flat column of keys far beyond a shared table: nearly every row would
+    // probe the shared table in vain (2.7 M int64 rows over 27 K uniform keys:
+    // 0.33 ms on shared tables, 0.27 ms on the global one)
+    if (q.strategy != AGG_STRAT_SMEM && est > 4.0 * maxs && key_estimate(f).flat) qp.strategy = AGG_STRAT_GLOBAL;
     const int64_t ss = next_pow2((int64_t)std::ceil(2.0 * est));
     qp.smem_slots = (int)std::max<int64_t>(256, std::min<int64_t>(ss, maxs));
     qp.cap = slots + 1;
     qp.large = qp.cap > kSmallRank;
   }
+  // Work items small enough that every resident block gets about four: one
+  // block folds an item's rows in a chain of loads and atomics (65532 float64
+  // rows over 128 K keys take it a millisecond), so a few large items leave
+  // the other blocks idle. Large batches keep 64 Ki rows (fewer merges).
+  int64_t rows = 0;
+  for (int i = 0; i < nq; ++i) rows += P->q[i].n;
+  P->tile_rows = kTileRows;
+  while (P->tile_rows > kMinTileRows && rows < 8 * (int64_t)device_info().sm_count * P->tile_rows) P->tile_rows >>= 1;
 }
 
 // Batched sketch and, with a selector installed, batched network inference.
@@ -758,7 +775,7 @@ static agg_status plan_retile(agg_batch_plan* P, int64_t tile_rows, cudaStream_t
   std::vector<int64_t> tp(P->nq + 1, 0);
   for (int i = 0; i < P->nq; ++i) {
     P->hq[i].tile0 = tp[i];
-    tp[i + 1] = tp[i] + (P->q[i].n + tile_rows - 1) / tile_rows;
+    tp[i + 1] = tp[i] + (P->q[i].n + item_rows(tile_rows) - 1) / item_rows(tile_rows);
   }
   P->total_tiles = tp[P->nq];
   if (P->nq > 0) {

@@ -96,19 +96,13 @@ static KernelPtr pick_build(int dt, bool mm, bool smem, bool vec, bool multi, in
   return nullptr;
 }
 
-template <int DT, bool MM>
-static KernelPtr tiles_kernel(int qpi, bool home) {
-  if (home)
-    return qpi == 2 ? (KernelPtr)gb_build_tiles<DT, MM, true, 2, true> : (KernelPtr)gb_build_tiles<DT, MM, true, 1, true>;
-  return qpi == 2 ? (KernelPtr)gb_build_tiles<DT, MM, true, 2> : (KernelPtr)gb_build_tiles<DT, MM, true, 1>;
-}
-
-// home: the tiles' shared tables are lightly loaded (see s_find_home).
-static KernelPtr pick_tiles(int dt, bool mm, int qpi, bool home) {
+static KernelPtr pick_tiles(int dt, bool mm, int qpi) {
+#define AGG_TK(D, M) (qpi == 2 ? (KernelPtr)gb_build_tiles<D, M, true, 2> : (KernelPtr)gb_build_tiles<D, M, true, 1>)
 #define AGG_T(D) \
-  case D: return mm ? tiles_kernel<D, true>(qpi, home) : tiles_kernel<D, false>(qpi, home);
+  case D: return mm ? AGG_TK(D, true) : AGG_TK(D, false);
   switch (dt) { AGG_T(AGG_I32) AGG_T(AGG_I64) AGG_T(AGG_U32) AGG_T(AGG_F32) AGG_T(AGG_F64) }
 #undef AGG_T
+#undef AGG_TK
   return nullptr;
 }
 
@@ -141,22 +135,6 @@ static KernelPtr pick_gather(int dt, bool mm) {
   return nullptr;
 }
 
-static size_t stab_bytes_dt(int dt, bool mm, int S) {
-#define AGG_SB(D) \
-  case D: return mm ? stab_bytes<D, true>(S) : stab_bytes<D, false>(S);
-  switch (dt) { AGG_SB(AGG_I32) AGG_SB(AGG_I64) AGG_SB(AGG_U32) AGG_SB(AGG_F32) AGG_SB(AGG_F64) }
-#undef AGG_SB
-  return 0;
-}
-
-static size_t tile_smem_bytes_dt(int dt, bool mm, int S) {
-#define AGG_SB(D) \
-  case D: return mm ? tile_smem_bytes<D, true>(S) : tile_smem_bytes<D, false>(S);
-  switch (dt) { AGG_SB(AGG_I32) AGG_SB(AGG_I64) AGG_SB(AGG_U32) AGG_SB(AGG_F32) AGG_SB(AGG_F64) }
-#undef AGG_SB
-  return 0;
-}
-
 // Resident blocks per SM of a kernel for (threads, dynamic smem), cached.
 static int occupancy(KernelPtr fn, int threads, size_t smem) {
   static std::mutex mu;
@@ -167,7 +145,12 @@ static int occupancy(KernelPtr fn, int threads, size_t smem) {
   auto key = std::make_tuple(dev, fn, threads, smem);
   auto it = cache.find(key);
   if (it != cache.end()) return it->second;
-  if (smem > 48 * 1024) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (smem > 48 * 1024) {  // the limit only rises: a larger table's cached entry relies on it
+    static std::map<std::pair<int, KernelPtr>, size_t> limit;
+    size_t& l = limit[{dev, fn}];
+    if (smem > l && cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess)
+      l = smem;
+  }
   int b = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fn, threads, smem) != cudaSuccess || b < 1) b = 1;
   cache[key] = b;
@@ -312,29 +295,17 @@ struct HashPlan {
   int64_t slots;    // global main slots (power of two)
   int smem_slots;   // shared slots (power of two) for SMEM
   int threads;
+  bool threads_given = false, smem_given = false;  // by the caller's options
   int blocks_per_sm;
   bool multi_keys = true;  // per-warp reduction of several frequent keys (see build_rows)
   // quads (4 rows) a thread folds per iteration: items per thread / 4; 0 = the
-  // default: 2 for the plain shared-memory build of integer columns without
-  // the frequent-key step (2^26 rows over 64-1024 uniform keys: up to 3 %
-  // faster; int64, 1024 keys: 0.401 vs 0.409 ms), else 1 (float columns
-  // measured up to 2 % slower with 2, the tile builds 1.5x slower)
+  // default, 1 (2^24 int64 rows over 1024 keys: 94 us with 1, 107 us with 2)
   int qpi = 0;
   int64_t tile_rows = 0;   // rows per tile of the partitioned build (0: from the column)
   // Rows of each one-level partition of the column (host memory, counted by
   // the HyperLogLog pass), or null: the partition then counts them itself.
   const unsigned long long* part_hist = nullptr;
-  double est_keys = 0.0;  // the planner's distinct-key estimate of the column
 };
-
-// Whether a partitioned build's shared tables stay lightly loaded (at most a
-// quarter of the slots): about est / P keys per tile when a tile lies within
-// one of the P partitions, proportionally more when it spans several.
-static bool tiles_lightly_loaded(double est, int64_t n, int passes, int64_t tile_rows, int smem_slots) {
-  const double parts = passes == 2 ? 65536.0 : 256.0;
-  const double span = std::max(1.0, (double)tile_rows * parts / (double)std::max<int64_t>(n, 1));
-  return est > 0.0 && (est / parts) * span <= 0.25 * (double)smem_slots;
-}
 
 // One hash aggregation: a zeroed global table, any number of build launches
 // over row ranges (one for a device column, one per chunk for a host-fed
@@ -386,20 +357,31 @@ class HashRun {
     a.table = mem_;
     a.mask = (uint32_t)(plan_.slots - 1);
     a.gshift = 32 - (63 - __builtin_clzll((unsigned long long)plan_.slots));
-    a.smem_slots = use_smem ? plan_.smem_slots : 0;
-    a.smem_cap = use_smem ? (plan_.smem_slots * 3) / 4 : 0;
     a.status = status_;
     a.progress = progress_;
-    if (plan_.partition && n >= kPartTileRows) return build_partitioned(a, use_smem);
-    const bool int_col = vdt_ == AGG_I32 || vdt_ == AGG_I64 || vdt_ == AGG_U32;
-    const int qpi = plan_.qpi ? plan_.qpi : (use_smem && !plan_.multi_keys && int_col ? 2 : 1);
+    const bool tiled = plan_.partition && n >= kPartTileRows;
+    if (use_smem) {
+      // the unpartitioned build has the SM's shared memory to itself: its table
+      // is loaded to a quarter at most where the plan sized it for a half
+      const int most = stab_max_slots(vdt_, mm_, !tiled);
+      if (!tiled && !plan_.smem_given) plan_.smem_slots *= 2;
+      plan_.smem_slots = std::min(plan_.smem_slots, most);
+    }
+    a.smem_slots = use_smem ? plan_.smem_slots : 0;
+    if (tiled) return build_partitioned(a, use_smem);
+    const int qpi = plan_.qpi ? plan_.qpi : 1;
     KernelPtr bk = pick_build(vdt_, mm_, use_smem, vec, plan_.multi_keys, qpi);
-    const size_t smem = use_smem ? tile_smem_bytes_dt(vdt_, mm_, plan_.smem_slots) : 0;  // table + 32-bit pairs
-    const int threads = plan_.threads;
-    int bps = occupancy(bk, threads, smem);
-    if (plan_.blocks_per_sm > 0 && plan_.blocks_per_sm < bps) bps = plan_.blocks_per_sm;
+    const size_t smem = use_smem ? stab_bytes_dt(vdt_, mm_, true) : 0;
+    // a table that leaves no room for a second block on the SM gets all its warps
+    int threads = plan_.threads;
     const DeviceInfo& di = device_info();
     const int64_t work = vec ? (n + 3) / 4 : n;
+    if (!plan_.threads_given && use_smem) {
+      if (smem > (size_t)di.smem_per_sm / 2 - 1280) threads = 1024;
+      while (threads > 256 && work < (int64_t)threads * di.sm_count) threads >>= 1;  // a small column: more blocks
+    }
+    int bps = occupancy(bk, threads, smem);
+    if (plan_.blocks_per_sm > 0 && plan_.blocks_per_sm < bps) bps = plan_.blocks_per_sm;
     int64_t grid = (int64_t)di.sm_count * bps;
     const int64_t need = (work + threads - 1) / threads;
     if (need < grid) grid = need < 1 ? 1 : need;
@@ -463,10 +445,10 @@ class HashRun {
           set_error("partitioned build: %s", cudaGetErrorString(e));
           return AGG_ERR_CUDA;
         }
-        const size_t smem = tile_smem_bytes_dt(vdt_, mm_, plan_.smem_slots);
+        const size_t smem = stab_bytes_dt(vdt_, mm_, false);
         const int threads = plan_.threads;
-        // both variants have the same resources: occupancy from either
-        int bps = occupancy(pick_tiles(vdt_, mm_, plan_.qpi, false), threads, smem);
+        KernelPtr bk = pick_tiles(vdt_, mm_, plan_.qpi);
+        int bps = occupancy(bk, threads, smem);
         if (plan_.blocks_per_sm > 0 && plan_.blocks_per_sm < bps) bps = plan_.blocks_per_sm;
         int64_t grid = (int64_t)di.sm_count * bps;
         // tiles of up to 65532 rows (32 Ki after two levels), smaller (down to
@@ -477,9 +459,6 @@ class HashRun {
           while (tile_rows > 4096 && n < 2 * grid * tile_rows) tile_rows >>= 1;
         }
         tile_rows = std::min(tile_rows, kTileRowsMax);
-        KernelPtr bk = pick_tiles(vdt_, mm_, plan_.qpi,
-                                  tiles_lightly_loaded(plan_.est_keys, n, passes, tile_rows, plan_.smem_slots));
-        (void)occupancy(bk, threads, smem);  // sets the kernel's shared-memory limit
         const int64_t tiles = (n + tile_rows - 1) / tile_rows;
         if (tiles < grid) grid = tiles;
         const longlong2* no_tiles = nullptr;
@@ -521,8 +500,8 @@ class HashRun {
     a.table = mem_;
     a.mask = (uint32_t)(plan_.slots - 1);
     a.gshift = 32 - (63 - __builtin_clzll((unsigned long long)plan_.slots));
+    plan_.smem_slots = std::min(plan_.smem_slots, stab_max_slots(vdt_, mm_, false));
     a.smem_slots = plan_.smem_slots;
-    a.smem_cap = (plan_.smem_slots * 3) / 4;
     a.status = status_;
     a.progress = progress_;
     int64_t tile_rows = std::min(plan_.tile_rows ? (int64_t)plan_.tile_rows : kPartTileRows / 2, kTileRowsMax);
@@ -531,8 +510,8 @@ class HashRun {
     note_launch();
     unsigned long long* next_tile = (unsigned long long*)((char*)mem_ + status_off_ + 128);
     AGG_CUDA_TRY(cudaMemsetAsync(next_tile, 0, 8, s_));
-    KernelPtr bk = pick_tiles(vdt_, mm_, plan_.qpi, tiles_lightly_loaded(plan_.est_keys, n, 1, 1, plan_.smem_slots));
-    const size_t smem = tile_smem_bytes_dt(vdt_, mm_, plan_.smem_slots);
+    KernelPtr bk = pick_tiles(vdt_, mm_, plan_.qpi);
+    const size_t smem = stab_bytes_dt(vdt_, mm_, false);
     int bps = occupancy(bk, plan_.threads, smem);
     if (plan_.blocks_per_sm > 0 && plan_.blocks_per_sm < bps) bps = plan_.blocks_per_sm;
     const int64_t grid = (int64_t)device_info().sm_count * bps;
@@ -759,7 +738,10 @@ static agg_status choose(const uint32_t* keys, const void* vals, int64_t n, int 
   c->plan.strategy = strategy;
   c->plan.slots = tslots ? tslots
                          : hll > 0.0 ? slots_for_count(hll, n) : (have_feat ? table_slots_from_sketch(feat, n) : 2048);
-  c->plan.smem_slots = sslots ? sslots : smem_slots_for(est, ops_minmax(ops));
+  c->plan.smem_slots = sslots ? std::min(sslots, stab_max_slots(vdt, ops_minmax(ops), true))
+                              : smem_slots_for(est, ops_minmax(ops));
+  c->plan.threads_given = o.block_threads != 0;
+  c->plan.smem_given = o.smem_slots != 0;
   c->plan.threads = o.block_threads ? o.block_threads : (strategy == AGG_STRAT_SMEM ? 512 : 256);
   // frequent keys (a key with >= 3% of the sample, or a handful of keys) make
   // the warp-level reduction of several keys pay; without a sketch, assume so
@@ -767,7 +749,6 @@ static agg_status choose(const uint32_t* keys, const void* vals, int64_t n, int 
   c->plan.blocks_per_sm = o.blocks_per_sm;
   c->plan.qpi = items == 8 ? 2 : items == 4 ? 1 : 0;
   c->plan.tile_rows = tile;
-  c->plan.est_keys = est;
   // Partition the rows by hash first when the shared tables would spill (more
   // distinct keys than a shared table admits) or the global table exceeds
   // half of L2; each partition then has about 1/256 of the keys.
