@@ -378,7 +378,7 @@ class HashRun {
     const int64_t work = vec ? (n + 3) / 4 : n;
     if (!plan_.threads_given && use_smem) {
       if (smem > (size_t)di.smem_per_sm / 2 - 1280) threads = 1024;
-      while (threads > 256 && work < (int64_t)threads * di.sm_count) threads >>= 1;  // a small column: more blocks
+      if (work < (int64_t)threads * di.sm_count) threads = 512;  // a small column: more blocks
     }
     int bps = occupancy(bk, threads, smem);
     if (plan_.blocks_per_sm > 0 && plan_.blocks_per_sm < bps) bps = plan_.blocks_per_sm;
@@ -530,8 +530,36 @@ class HashRun {
   // Finalise into a new result; TABLE_FULL (and no result) if the table overflowed.
   agg_status finish(agg_groups** gout) {
     *gout = nullptr;
+    uint32_t mask = (uint32_t)(plan_.slots - 1);
+    const DeviceInfo& di = device_info();
+    PhaseTimer pt(AGG_PHASE_FINALIZE, s_);
+    char* aux = (char*)mem_ + aux_off_;
+    uint32_t* k0 = (uint32_t*)aux;  // the occupied slots' keys and slot numbers
+    uint32_t* s0 = k0 + nslots_;
+    if (small_) {
+      const int cgrid = (int)((nslots_ + 255) / 256);
+      if (mm_) gb_compact<true, 1><<<cgrid, 256, 0, s_>>>((const GSlot<true>*)mem_, mask, k0, s0, counter_);
+      else gb_compact<false, 1><<<cgrid, 256, 0, s_>>>((const GSlot<false>*)mem_, mask, k0, s0, counter_);
+    } else {
+      const int64_t cgrid = std::min<int64_t>((nslots_ + 255) / 256, (int64_t)di.sm_count * 8);
+      if (mm_) gb_compact<true><<<(unsigned)cgrid, 256, 0, s_>>>((const GSlot<true>*)mem_, mask, k0, s0, counter_);
+      else gb_compact<false><<<(unsigned)cgrid, 256, 0, s_>>>((const GSlot<false>*)mem_, mask, k0, s0, counter_);
+    }
+    note_launch();
+    // A large table's group count is read back here, so that the result, the
+    // sort and the gather are sized by the groups and not by the slots: a
+    // result of 33 M slots (1.5 GB for 14 M groups) also made every call whose
+    // previous result was still held move memory in the allocation pool (2.5
+    // ms a call).
+    const bool counted = nslots_ > kCountSlots;
+    agg_status st = AGG_OK;
+    int64_t d = nslots_;  // groups, at most
+    if (counted) {
+      st = read_back(&d);
+      if (st != AGG_OK) return st;
+    }
     agg_groups* g = nullptr;
-    agg_status st = groups_alloc(nslots_, vdt_, ops_, s_, &g);
+    st = groups_alloc(d, vdt_, ops_, s_, &g);
     if (st != AGG_OK) return st;
     OutArrays o;
     o.keys = g->keys;
@@ -541,43 +569,25 @@ class HashRun {
     o.max = (unsigned long long*)g->max;
     o.avg = g->avg;
     o.d = (int64_t*)counter_;
-    uint32_t mask = (uint32_t)(plan_.slots - 1);
-    const DeviceInfo& di = device_info();
     cudaError_t e;
-    PhaseTimer pt(AGG_PHASE_FINALIZE, s_);
     if (small_) {
-      char* aux = (char*)mem_ + aux_off_;
-      uint32_t* ck = (uint32_t*)aux;
-      uint32_t* cs = ck + nslots_;
-      const int cgrid = (int)((nslots_ + 255) / 256);
-      if (mm_) gb_compact<true, 1><<<cgrid, 256, 0, s_>>>((const GSlot<true>*)mem_, mask, ck, cs, counter_);
-      else gb_compact<false, 1><<<cgrid, 256, 0, s_>>>((const GSlot<false>*)mem_, mask, ck, cs, counter_);
-      note_launch();
       const int rgrid = (int)((nslots_ + kRankKeys - 1) / kRankKeys);
-      void* args[] = {&mem_, &ck, &cs, &o};
+      void* args[] = {&mem_, &k0, &s0, &o};
       e = cudaLaunchKernel(pick_small(vdt_, mm_), dim3(rgrid), dim3(kRankThreads), args, 0, s_);
       note_launch();
     } else {
-      char* aux = (char*)mem_ + aux_off_;
-      uint32_t* k0 = (uint32_t*)aux;
-      uint32_t* s0 = k0 + nslots_;
       uint32_t* k1 = s0 + nslots_;
       uint32_t* s1 = k1 + nslots_;
       void* rtmp = (void*)(((uintptr_t)(s1 + nslots_) + 255) & ~(uintptr_t)255);
-      int64_t cgrid = (nslots_ + 255) / 256;
-      if (cgrid > (int64_t)di.sm_count * 8) cgrid = (int64_t)di.sm_count * 8;
-      if (mm_) gb_compact<true><<<(unsigned)cgrid, 256, 0, s_>>>((const GSlot<true>*)mem_, mask, k0, s0, counter_);
-      else gb_compact<false><<<(unsigned)cgrid, 256, 0, s_>>>((const GSlot<false>*)mem_, mask, k0, s0, counter_);
-      note_launch();
       uint32_t *sk = nullptr, *ss = nullptr;
-      st = radix_sort_pairs<uint32_t>(k0, s0, k1, s1, k0, s0, nslots_, (const int64_t*)counter_, 32, rtmp, s_,
-                                      &sk, &ss);
+      st = radix_sort_pairs<uint32_t>(k0, s0, k1, s1, k0, s0, d, counted ? nullptr : (const int64_t*)counter_, 32,
+                                      rtmp, s_, &sk, &ss);
       if (st != AGG_OK) {
         agg_groups_free(g);
         return st;
       }
-      int64_t ggrid = cgrid;
-      int64_t cap = nslots_;
+      const int64_t ggrid = std::max<int64_t>(1, std::min<int64_t>((d + 255) / 256, (int64_t)di.sm_count * 8));
+      int64_t cap = d;
       void* args[] = {&mem_, &sk, &ss, &o, &cap};
       e = cudaLaunchKernel(pick_gather(vdt_, mm_), dim3((unsigned)ggrid), dim3(256), args, 0, s_);
       note_launch();
@@ -587,29 +597,21 @@ class HashRun {
       agg_groups_free(g);
       return AGG_ERR_CUDA;
     }
-    // one copy of the status block: status (+0), group count (+64), and the
-    // rows seen / failed of a build stopped by a full table (+192, +200)
-    unsigned char* hb = (unsigned char*)stream_pinned(s_, 256, &st);
-    if (!hb) {
-      agg_groups_free(g);
-      return st;
+    if (counted) {
+      const cudaError_t es = cudaStreamSynchronize(s_);
+      if (es != cudaSuccess) {
+        set_error("group-by finalize failed: %s", cudaGetErrorString(es));
+        agg_groups_free(g);
+        return AGG_ERR_CUDA;
+      }
+    } else {
+      st = read_back(&d);
+      if (st != AGG_OK) {
+        agg_groups_free(g);
+        return st;
+      }
     }
-    const cudaError_t e1 = cudaMemcpyAsync(hb, status_, 208, cudaMemcpyDeviceToHost, s_);
-    const cudaError_t e3 = cudaStreamSynchronize(s_);
-    if (e1 != cudaSuccess || e3 != cudaSuccess) {
-      set_error("group-by read-back failed: %s", cudaGetErrorString(e3 != cudaSuccess ? e3 : e1));
-      agg_groups_free(g);
-      return AGG_ERR_CUDA;
-    }
-    const int64_t groups = *(const int64_t*)(hb + 64);
-    if (*(const int*)hb != 0) {
-      rows_seen_ = *(const uint64_t*)(hb + 192);
-      rows_failed_ = *(const uint64_t*)(hb + 200);
-      agg_groups_free(g);
-      set_error("global hash table of %lld slots is full", (long long)plan_.slots);
-      return AGG_ERR_TABLE_FULL;
-    }
-    g->num_groups = groups;
+    g->num_groups = d;
     g->table_slots = plan_.slots;
     g->smem_slots = plan_.strategy == AGG_STRAT_SMEM ? plan_.smem_slots : 0;
     g->strategy = plan_.strategy;
@@ -618,6 +620,31 @@ class HashRun {
   }
 
  private:
+  static constexpr int64_t kCountSlots = int64_t(1) << 20;
+
+  // One copy of the status block: status (+0), group count (+64), and the rows
+  // seen / failed of a build stopped by a full table (+192, +200). Waits for
+  // the stream; TABLE_FULL if the table overflowed.
+  agg_status read_back(int64_t* groups) {
+    agg_status st = AGG_OK;
+    unsigned char* hb = (unsigned char*)stream_pinned(s_, 256, &st);
+    if (!hb) return st;
+    const cudaError_t e1 = cudaMemcpyAsync(hb, status_, 208, cudaMemcpyDeviceToHost, s_);
+    const cudaError_t e3 = cudaStreamSynchronize(s_);
+    if (e1 != cudaSuccess || e3 != cudaSuccess) {
+      set_error("group-by read-back failed: %s", cudaGetErrorString(e3 != cudaSuccess ? e3 : e1));
+      return AGG_ERR_CUDA;
+    }
+    *groups = *(const int64_t*)(hb + 64);
+    if (*(const int*)hb != 0) {
+      rows_seen_ = *(const uint64_t*)(hb + 192);
+      rows_failed_ = *(const uint64_t*)(hb + 200);
+      set_error("global hash table of %lld slots is full", (long long)plan_.slots);
+      return AGG_ERR_TABLE_FULL;
+    }
+    return AGG_OK;
+  }
+
   int vdt_;
   uint32_t ops_;
   bool mm_;

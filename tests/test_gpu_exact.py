@@ -164,3 +164,22 @@ def test_sum_error_is_absent_for_integer_columns():
                         agg.options(flags=agg.AGG_FLAG_SUM_ERROR))
     assert not g.has_sum_err
     g.free()
+
+
+@pytest.mark.parametrize("dt", ["f32", "f64"])
+@pytest.mark.parametrize("keys,n,kind", [(1, 5, "default"), (3, 12_000_011, "default"), (3000, 800_001, "default"),
+                                         (3000, 800_001, "span"), (9000, 2_400_003, "default")])
+def test_exact_sums_added_in_shared_memory(dt, keys, n, kind):
+    """One group, blocks that carry their digits several times, as many groups as a block holds (and
+    more), and an exponent span whose digits just fit: bit-identical to the oracle."""
+    k = dg.keys_uniform(n, keys, 21)
+    v = dg.values(dt, n, 22)
+    if kind == "span":
+        v = (v * np.exp2(np.random.default_rng(1).integers(-60, 60, n).astype(np.float64))).astype(NP[dt])
+    if keys > 1:
+        k[::101] = 0xFFFFFFFF
+    res = run(k, v, agg.AGG_STRAT_AUTO)
+    ref = oracle.groupby(k, v)
+    assert np.array_equal(res["keys"], ref.keys) and np.array_equal(res["count"], ref.count)
+    assert np.array_equal(res["sum"].view(np.int64), ref.sum.view(np.int64))
+    assert np.array_equal(res["avg"].view(np.int64), ref.avg.view(np.int64))
