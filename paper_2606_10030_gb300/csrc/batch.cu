@@ -49,6 +49,7 @@ struct BQ {  // one query of a batch, on the device
   int* status;
   int64_t slot0;  // first slot of this query in the concatenated large-table slot space (-1: small)
   OutArrays out;
+  double* avg;  // the result's array (out.avg is null when neither SUM nor AVG was asked for)
   uint32_t mask;
   int dt, mm, smem, vec;
   int smem_slots;
@@ -167,8 +168,8 @@ __device__ void small_finalize(const BQ& q, uint32_t* ck, uint32_t* cs, int* s_d
 
 __global__ void __launch_bounds__(kFinThreads) batch_finalize_small(const BQ* __restrict__ qs,
                                                                     const int* __restrict__ small_ids) {
-  __shared__ uint32_t ck[kSmallRank];
-  __shared__ uint32_t cs[kSmallRank];
+  __shared__ uint32_t ck[kSmallSlots];
+  __shared__ uint32_t cs[kSmallSlots];
   __shared__ int s_d;
   if (threadIdx.x == 0) s_d = 0;
   __syncthreads();
@@ -475,7 +476,8 @@ static agg_status plan_alloc(agg_batch_plan* P, cudaStream_t s) {
     o += align256((size_t)cap * 8);
     b.out.max = (unsigned long long*)o;
     o += align256((size_t)cap * 8);
-    b.out.avg = (double*)o;
+    b.avg = (double*)o;
+    b.out.avg = (q.ops & (AGG_SUM | AGG_AVG)) ? b.avg : nullptr;
     b.out.d = P->dcount + i;
     if (b.smem) {
       const size_t sb = stab_bytes_dt(b.dt, b.mm, false);
@@ -608,7 +610,7 @@ static void plan_sizes(agg_batch_plan* P, const std::vector<int>& learned) {
     const int64_t ss = next_pow2((int64_t)std::ceil(2.0 * est));
     qp.smem_slots = (int)std::max<int64_t>(256, std::min<int64_t>(ss, maxs));
     qp.cap = slots + 1;
-    qp.large = qp.cap > kSmallRank;
+    qp.large = qp.cap > kSmallSlots;
   }
   // Work items small enough that every resident block gets about four: one
   // block folds an item's rows in a chain of loads and atomics (65532 float64
@@ -749,7 +751,7 @@ extern "C" agg_status agg_batch_run(agg_batch_plan* P, void* stream) {
         any_full = true;
         P->qp[i].slots = std::min<int64_t>(P->qp[i].slots * 4, int64_t(1) << 31);
         P->qp[i].cap = P->qp[i].slots + 1;
-        P->qp[i].large = P->qp[i].cap > kSmallRank;
+        P->qp[i].large = P->qp[i].cap > kSmallSlots;
       }
     }
     if (!any_full) return AGG_OK;
@@ -844,7 +846,7 @@ extern "C" agg_status agg_batch_result(const agg_batch_plan* P, int i, agg_group
   g->sum = b.out.sum;
   g->min = b.out.min;
   g->max = b.out.max;
-  g->avg = b.out.avg;
+  g->avg = b.avg;
   std::memcpy(g->features, &P->features[(size_t)i * F_COUNT], sizeof(float) * F_COUNT);
   auto* priv = new GroupsPriv();
   priv->block = nullptr;

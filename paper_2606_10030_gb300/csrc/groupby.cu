@@ -106,34 +106,21 @@ static KernelPtr pick_tiles(int dt, bool mm, int qpi) {
   return nullptr;
 }
 
-template <int DT>
-static KernelPtr fin_small(bool mm) {
-  return mm ? (KernelPtr)gb_rank_gather<DT, true> : (KernelPtr)gb_rank_gather<DT, false>;
-}
-template <int DT>
-static KernelPtr fin_gather(bool mm) {
-  return mm ? (KernelPtr)gb_gather<DT, true> : (KernelPtr)gb_gather<DT, false>;
-}
-static KernelPtr pick_small(int dt, bool mm) {
-  switch (dt) {
-    case AGG_I32: return fin_small<AGG_I32>(mm);
-    case AGG_I64: return fin_small<AGG_I64>(mm);
-    case AGG_U32: return fin_small<AGG_U32>(mm);
-    case AGG_F32: return fin_small<AGG_F32>(mm);
-    case AGG_F64: return fin_small<AGG_F64>(mm);
+#define AGG_PICK(name, kernel)                                                         \
+  static KernelPtr name(int dt, bool mm) {                                             \
+    switch (dt) {                                                                      \
+      case AGG_I32: return mm ? (KernelPtr)kernel<AGG_I32, true> : (KernelPtr)kernel<AGG_I32, false>; \
+      case AGG_I64: return mm ? (KernelPtr)kernel<AGG_I64, true> : (KernelPtr)kernel<AGG_I64, false>; \
+      case AGG_U32: return mm ? (KernelPtr)kernel<AGG_U32, true> : (KernelPtr)kernel<AGG_U32, false>; \
+      case AGG_F32: return mm ? (KernelPtr)kernel<AGG_F32, true> : (KernelPtr)kernel<AGG_F32, false>; \
+      case AGG_F64: return mm ? (KernelPtr)kernel<AGG_F64, true> : (KernelPtr)kernel<AGG_F64, false>; \
+    }                                                                                  \
+    return nullptr;                                                                    \
   }
-  return nullptr;
-}
-static KernelPtr pick_gather(int dt, bool mm) {
-  switch (dt) {
-    case AGG_I32: return fin_gather<AGG_I32>(mm);
-    case AGG_I64: return fin_gather<AGG_I64>(mm);
-    case AGG_U32: return fin_gather<AGG_U32>(mm);
-    case AGG_F32: return fin_gather<AGG_F32>(mm);
-    case AGG_F64: return fin_gather<AGG_F64>(mm);
-  }
-  return nullptr;
-}
+AGG_PICK(pick_small, gb_rank_small)
+AGG_PICK(pick_rank, gb_rank_gather)
+AGG_PICK(pick_gather, gb_gather)
+#undef AGG_PICK
 
 // Resident blocks per SM of a kernel for (threads, dynamic smem), cached.
 static int occupancy(KernelPtr fn, int threads, size_t smem) {
@@ -321,11 +308,12 @@ class HashRun {
   agg_status init() {
     const size_t slot = (size_t)gslot_bytes(mm_);
     nslots_ = plan_.slots + 1;
-    small_ = nslots_ <= kSmallRank;
+    small_ = nslots_ <= kSmallSlots;
+    ranked_ = !small_ && nslots_ <= kRankSlots;
     const size_t tbytes = (size_t)(nslots_ + 1) * slot;
     status_off_ = (tbytes + 255) & ~size_t(255);
     aux_off_ = status_off_ + 256;
-    size_t aux_bytes = small_ ? 2 * (size_t)nslots_ * 4 + 1024 : 4 * (size_t)nslots_ * 4 + 1024 + radix_tmp_bytes(nslots_);
+    size_t aux_bytes = small_ || ranked_ ? 2 * (size_t)nslots_ * 4 + 1024 : 4 * (size_t)nslots_ * 4 + 1024 + radix_tmp_bytes(nslots_);
     AGG_CUDA_TRY(dev_malloc_async(&mem_, aux_off_ + aux_bytes, s_));
     AGG_CUDA_TRY(cudaMemsetAsync(mem_, 0, aux_off_, s_));
     status_ = (int*)((char*)mem_ + status_off_);
@@ -536,16 +524,17 @@ class HashRun {
     char* aux = (char*)mem_ + aux_off_;
     uint32_t* k0 = (uint32_t*)aux;  // the occupied slots' keys and slot numbers
     uint32_t* s0 = k0 + nslots_;
-    if (small_) {
-      const int cgrid = (int)((nslots_ + 255) / 256);
-      if (mm_) gb_compact<true, 1><<<cgrid, 256, 0, s_>>>((const GSlot<true>*)mem_, mask, k0, s0, counter_);
-      else gb_compact<false, 1><<<cgrid, 256, 0, s_>>>((const GSlot<false>*)mem_, mask, k0, s0, counter_);
-    } else {
+    if (!small_) {
       const int64_t cgrid = std::min<int64_t>((nslots_ + 255) / 256, (int64_t)di.sm_count * 8);
-      if (mm_) gb_compact<true><<<(unsigned)cgrid, 256, 0, s_>>>((const GSlot<true>*)mem_, mask, k0, s0, counter_);
-      else gb_compact<false><<<(unsigned)cgrid, 256, 0, s_>>>((const GSlot<false>*)mem_, mask, k0, s0, counter_);
+      if (ranked_) {
+        if (mm_) gb_compact<true, 1><<<(unsigned)cgrid, 256, 0, s_>>>((const GSlot<true>*)mem_, mask, k0, s0, counter_);
+        else gb_compact<false, 1><<<(unsigned)cgrid, 256, 0, s_>>>((const GSlot<false>*)mem_, mask, k0, s0, counter_);
+      } else {
+        if (mm_) gb_compact<true><<<(unsigned)cgrid, 256, 0, s_>>>((const GSlot<true>*)mem_, mask, k0, s0, counter_);
+        else gb_compact<false><<<(unsigned)cgrid, 256, 0, s_>>>((const GSlot<false>*)mem_, mask, k0, s0, counter_);
+      }
+      note_launch();
     }
-    note_launch();
     // A large table's group count is read back here, so that the result, the
     // sort and the gather are sized by the groups and not by the slots: a
     // result of 33 M slots (1.5 GB for 14 M groups) also made every call whose
@@ -567,13 +556,20 @@ class HashRun {
     o.sum = (unsigned long long*)g->sum;
     o.min = (unsigned long long*)g->min;
     o.max = (unsigned long long*)g->max;
-    o.avg = g->avg;
+    o.avg = (ops_ & (AGG_SUM | AGG_AVG)) ? g->avg : nullptr;
     o.d = (int64_t*)counter_;
     cudaError_t e;
+    const unsigned rgrid = (unsigned)((nslots_ + kRankKeys - 1) / kRankKeys);
     if (small_) {
-      const int rgrid = (int)((nslots_ + kRankKeys - 1) / kRankKeys);
-      void* args[] = {&mem_, &k0, &s0, &o};
+      void* args[] = {&mem_, &mask, &o};
       e = cudaLaunchKernel(pick_small(vdt_, mm_), dim3(rgrid), dim3(kRankThreads), args, 0, s_);
+      note_launch();
+    } else if (ranked_) {
+      KernelPtr rk = pick_rank(vdt_, mm_);
+      const size_t sm = ((size_t)nslots_ + 4) * 4;
+      (void)occupancy(rk, kRankThreads, sm);  // sets the kernel's shared-memory limit
+      void* args[] = {&mem_, &k0, &s0, &o};
+      e = cudaLaunchKernel(rk, dim3(rgrid), dim3(kRankThreads), args, sm, s_);
       note_launch();
     } else {
       uint32_t* k1 = s0 + nslots_;
@@ -652,7 +648,7 @@ class HashRun {
   cudaStream_t s_;
   void* mem_ = nullptr;
   int64_t nslots_ = 0;
-  bool small_ = true;
+  bool small_ = true, ranked_ = false;
   size_t status_off_ = 0, aux_off_ = 0;
   int* status_ = nullptr;
   unsigned long long* progress_ = nullptr;

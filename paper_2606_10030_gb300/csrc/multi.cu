@@ -23,6 +23,7 @@
 #include <cstring>
 
 #include "groupby.cuh"
+#include "quotient.cuh"
 #include "sort.cuh"
 
 namespace agg {
@@ -48,6 +49,7 @@ struct MultiArgs {
   const void* col[AGG_MAX_COLUMNS];
   int dt[AGG_MAX_COLUMNS];
   bool mm[AGG_MAX_COLUMNS];
+  bool avg[AGG_MAX_COLUMNS];
   const void* fcol;  // null: no filter
   int fdt;
   int64_t flo_i, fhi_i;
@@ -292,8 +294,9 @@ __global__ void multi_gather(MultiArgs a, const uint32_t* slot, const uint32_t* 
       const unsigned long long sv = a.sum[c][j];
       const bool fp = a.dt[c] == AGG_F32 || a.dt[c] == AGG_F64;
       o.sum[c][i] = sv;
-      const double s = fp ? __longlong_as_double((long long)sv) : (double)(long long)sv;
-      o.avg[c][i] = s / (double)c0;
+      if (a.avg[c]) {
+        o.avg[c][i] = average(fp ? sv : float64_bits_of((long long)sv), c0);
+      }
       if (a.mm[c]) {
         const uint64_t mn = ~a.minc[c][j], mx = a.mx[c][j];
         if (fp) {
@@ -515,6 +518,7 @@ extern "C" agg_status agg_groupby_multi(const uint32_t* key_lo_dev, const uint32
     a.col[c] = cols[c].data;
     a.dt[c] = cols[c].dtype;
     a.mm[c] = ops_minmax(cols[c].ops);
+    a.avg[c] = (cols[c].ops & (AGG_SUM | AGG_AVG)) != 0;
   }
   if (filter) {
     a.fcol = filter->data;

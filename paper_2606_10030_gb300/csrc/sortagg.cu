@@ -15,12 +15,12 @@
 //    cleared, the pieces added with atomics (one set per run per warp), and
 //    the targets brought to the raw form of the finished runs.
 // 5. seg_finalize converts every group to the output encodings and computes
-//    AVG in float64 with converged warps (GB300's float64 pipe is narrow; in
-//    the divergent per-run code it was the bottleneck).
+//    AVG with converged warps.
 // Runs come out in ascending key order by construction.
 #include <type_traits>
 
 #include "groupby.cuh"
+#include "quotient.cuh"
 #include "sort.cuh"
 
 namespace agg {
@@ -162,7 +162,7 @@ struct SegOut {
   unsigned long long* sum;
   unsigned long long* min;
   unsigned long long* max;
-  double* avg;
+  double* avg;  // null: neither SUM nor AVG asked for
 };
 
 // Part of a run cut by a chunk boundary.
@@ -445,14 +445,16 @@ __global__ void seg_piece_finish(const SegPiece* __restrict__ pieces, int64_t np
   }
 }
 
-// Every group: the output encodings and AVG = SUM / COUNT in float64.
+// Every group: the output encodings and AVG = SUM / COUNT.
 template <int DT, bool MM>
 __global__ void seg_finalize(SegOut o, int64_t d) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < d; i += (int64_t)gridDim.x * blockDim.x) {
-    const unsigned long long c = o.count[i];
-    const double fs = fsum_of_raw<DT>(o.sum[i]);
-    if (DT == AGG_F32) o.sum[i] = (unsigned long long)__double_as_longlong(fs);
-    o.avg[i] = fs / (double)c;
+    if (DT == AGG_F32 || o.avg) {
+      unsigned long long f = o.sum[i];  // the sum's float64 bits
+      if (DT == AGG_F32) o.sum[i] = f = (unsigned long long)__double_as_longlong(fsum_of_raw<DT>(f));
+      else if (DT != AGG_F64) f = float64_bits_of((long long)f);
+      if (o.avg) o.avg[i] = average(f, (uint32_t)o.count[i]);
+    }
     if (MM) {
       o.min[i] = out_of_img<DT>(o.min[i]);
       o.max[i] = out_of_img<DT>(o.max[i]);
@@ -579,7 +581,7 @@ static agg_status sort_groupby_t(const uint32_t* keys, const void* vals, int64_t
   o.sum = (unsigned long long*)g->sum;
   o.min = (unsigned long long*)g->min;
   o.max = (unsigned long long*)g->max;
-  o.avg = g->avg;
+  o.avg = (ops & (AGG_SUM | AGG_AVG)) ? g->avg : nullptr;
   seg_reduce<DT, MM><<<(unsigned)nblocks, kSegThreads, 0, s>>>(sk, sv, n, chunk_first, o, pieces);
   const DeviceInfo& di = device_info();
   int64_t pg = (np + 255) / 256;
@@ -591,8 +593,11 @@ static agg_status sort_groupby_t(const uint32_t* keys, const void* vals, int64_t
   int64_t fg = (d + 255) / 256;
   if (fg > (int64_t)di.sm_count * 8) fg = (int64_t)di.sm_count * 8;
   if (fg < 1) fg = 1;
-  seg_finalize<DT, MM><<<(unsigned)fg, 256, 0, s>>>(o, d);
-  note_launch(5);
+  note_launch(4);
+  if (MM || DT == AGG_F32 || o.avg) {  // counts and other sums are already as they go out
+    seg_finalize<DT, MM><<<(unsigned)fg, 256, 0, s>>>(o, d);
+    note_launch();
+  }
   e = cudaGetLastError();
   release();
   cudaError_t e2 = cudaStreamSynchronize(s);
