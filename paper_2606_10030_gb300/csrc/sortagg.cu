@@ -11,9 +11,10 @@
 //    with one segmented scan over the warp, and the run a lane's first head
 //    ends is written by that lane. The part of a run that crosses the chunk's
 //    start or end is written as a piece (at most two per chunk).
-// 4. The pieces of one run are consecutive in chunk order: their targets are
-//    cleared, the pieces added with atomics (one set per run per warp), and
-//    the targets brought to the raw form of the finished runs.
+// 4. The pieces of one run are consecutive in chunk order: their target is
+//    cleared by the chunk the run begins in, the pieces added with atomics (one
+//    set per run per warp), and the targets brought to the raw form of the
+//    finished runs.
 // 5. seg_finalize converts every group to the output encodings and computes
 //    AVG with converged warps.
 // Runs come out in ascending key order by construction.
@@ -353,24 +354,16 @@ __global__ void __launch_bounds__(kSegThreads) seg_reduce(const uint32_t* __rest
       pieces[2 * chunk + 1].run = kNoRun;
     } else {
       store_piece<DT, MM>(&pieces[2 * chunk + 1], run, last_key, xl);
+      if (heads_in_chunk > 0) {  // the run begins here: clear its target for the pieces (one chunk does)
+        o.count[run] = 0;
+        o.sum[run] = 0;
+        if (MM) {
+          o.min[run] = 0;
+          o.max[run] = 0;
+        }
+      }
     }
     if (!wrote_first) pieces[2 * chunk].run = kNoRun;
-  }
-}
-
-// Targets of pieces: clear count and sum, set MIN/MAX accumulators (the
-// complement of the MIN image and the MAX image, both combined with atomicMax).
-template <bool MM>
-__global__ void seg_piece_clear(const SegPiece* __restrict__ pieces, int64_t np, SegOut o) {
-  for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < np; p += (int64_t)gridDim.x * blockDim.x) {
-    const uint32_t run = pieces[p].run;
-    if (run == kNoRun) continue;
-    o.count[run] = 0;
-    o.sum[run] = 0;
-    if (MM) {
-      o.min[run] = 0;
-      o.max[run] = 0;
-    }
   }
 }
 
@@ -587,13 +580,12 @@ static agg_status sort_groupby_t(const uint32_t* keys, const void* vals, int64_t
   int64_t pg = (np + 255) / 256;
   if (pg > (int64_t)di.sm_count * 8) pg = (int64_t)di.sm_count * 8;
   if (pg < 1) pg = 1;
-  seg_piece_clear<MM><<<(unsigned)pg, 256, 0, s>>>(pieces, np, o);
   seg_piece_add<DT, MM><<<(unsigned)pg, 256, 0, s>>>(pieces, np, o);
   seg_piece_finish<DT, MM><<<(unsigned)pg, 256, 0, s>>>(pieces, np, o);
   int64_t fg = (d + 255) / 256;
   if (fg > (int64_t)di.sm_count * 8) fg = (int64_t)di.sm_count * 8;
   if (fg < 1) fg = 1;
-  note_launch(4);
+  note_launch(3);
   if (MM || DT == AGG_F32 || o.avg) {  // counts and other sums are already as they go out
     seg_finalize<DT, MM><<<(unsigned)fg, 256, 0, s>>>(o, d);
     note_launch();
