@@ -535,18 +535,20 @@ class HashRun {
       }
       note_launch();
     }
-    // A large table's group count is read back here, so that the result, the
-    // sort and the gather are sized by the groups and not by the slots: a
-    // result of 33 M slots (1.5 GB for 14 M groups) also made every call whose
-    // previous result was still held move memory in the allocation pool (2.5
-    // ms a call).
-    const bool counted = nslots_ > kCountSlots;
+    // The group count of a table too large to rank by its slots is read back
+    // here, so that the result, the ranking or sort and the gather are sized by
+    // the groups and not by the slots: 3 M rows over 10^4 Zipf keys in 2^20
+    // slots finalise in 61 us (104 us sorted by slots), and a result of 33 M
+    // slots (1.5 GB for 14 M groups) made every call whose previous result was
+    // still held move memory in the allocation pool (2.5 ms a call).
+    const bool counted = nslots_ > kRankSlots;
     agg_status st = AGG_OK;
     int64_t d = nslots_;  // groups, at most
     if (counted) {
       st = read_back(&d);
       if (st != AGG_OK) return st;
     }
+    const bool ranked = !small_ && d <= kRankSlots;
     agg_groups* g = nullptr;
     st = groups_alloc(d, vdt_, ops_, s_, &g);
     if (st != AGG_OK) return st;
@@ -559,14 +561,14 @@ class HashRun {
     o.avg = (ops_ & (AGG_SUM | AGG_AVG)) ? g->avg : nullptr;
     o.d = (int64_t*)counter_;
     cudaError_t e;
-    const unsigned rgrid = (unsigned)((nslots_ + kRankKeys - 1) / kRankKeys);
+    const unsigned rgrid = (unsigned)std::max<int64_t>(1, (d + kRankKeys - 1) / kRankKeys);
     if (small_) {
       void* args[] = {&mem_, &mask, &o};
       e = cudaLaunchKernel(pick_small(vdt_, mm_), dim3(rgrid), dim3(kRankThreads), args, 0, s_);
       note_launch();
-    } else if (ranked_) {
+    } else if (ranked) {
       KernelPtr rk = pick_rank(vdt_, mm_);
-      const size_t sm = ((size_t)nslots_ + 4) * 4;
+      const size_t sm = ((size_t)d + 4) * 4;
       (void)occupancy(rk, kRankThreads, sm);  // sets the kernel's shared-memory limit
       void* args[] = {&mem_, &k0, &s0, &o};
       e = cudaLaunchKernel(rk, dim3(rgrid), dim3(kRankThreads), args, sm, s_);
@@ -616,8 +618,6 @@ class HashRun {
   }
 
  private:
-  static constexpr int64_t kCountSlots = int64_t(1) << 20;
-
   // One copy of the status block: status (+0), group count (+64), and the rows
   // seen / failed of a build stopped by a full table (+192, +200). Waits for
   // the stream; TABLE_FULL if the table overflowed.
@@ -661,8 +661,7 @@ class HashRun {
 agg_status sort_groupby(const uint32_t* keys, const void* vals, int64_t n, int vdt, uint32_t ops, cudaStream_t s,
                         agg_groups** gout, const float* feat);
 
-static int smem_slots_for(double est, bool mm) {
-  const int maxs = mm ? 2048 : 4096;
+static int smem_slots_for(double est, int maxs) {
   int64_t s = next_pow2((int64_t)std::ceil(2.0 * est));
   if (s < 256) s = 256;
   if (s > maxs) s = maxs;
