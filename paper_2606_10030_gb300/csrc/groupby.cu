@@ -201,15 +201,22 @@ int64_t table_slots_from_sketch(const float* f, int64_t n) {
   return p;
 }
 
-// The AUTO rule (thresholds from the autotuner's timings of 5000 labelled
-// queries; m = 4096 sampled keys, coverage = 1 - f1 / m):
-//  - the sample covers >= 97% of the mass: SMEM (partitioned when the keys
-//    overflow a shared table);
+// The AUTO rule (m = 4096 sampled keys, coverage = 1 - f1 / m; calls timed on
+// int32 SUM/COUNT/MIN/MAX and float64 SUM/COUNT columns of 2^20 to 2^26 rows,
+// 3000 to 10^6 keys, uniform and Zipf 0.5 to 1.3; SMEM includes its partition):
+//  - the sample covers >= 97% of the mass: SMEM;
+//  - with the column's HyperLogLog count (2^22 rows and more): SMEM, from 2^24
+//    rows on (2^24 rows: 0.30-0.82 ms against 0.73-0.93 ms sorted) or while a
+//    key has 16 rows or more (below, the sort is up to 1.4x faster: 3 M rows
+//    over 950 K keys 0.32 ms against 0.44); flat columns of more than 2^25 keys
+//    sort (on 2^30 rows: 2^26 keys 45 ms sorted, 59 ms partitioned);
 //  - columns under 2^20 rows: SMEM for few keys or a skewed sample, else one
 //    global table;
-//  - a skewed sample covering 90-97% whose singletons suggest at least half
-//    as many unseen keys as seen ones (f1^2 / 2 f2 >= d / 2: a hot head and a
-//    long tail of rare keys): SORT, which needs no key count;
+//  - a skewed sample covering 70% of a column under 2^22 rows: SMEM (3 M rows
+//    over 10^4 Zipf 1 keys: 0.24 ms against 0.27 sorted; at 60% the two are
+//    level, at 48% 0.36 ms against 0.29); from 2^22 rows on, without the count
+//    (a batch), a skewed sample covering 90-97% whose singletons suggest at
+//    least half as many unseen keys as seen ones (f1^2 / 2 f2 >= d / 2) sorts;
 //  - few keys: SMEM;
 //  - a flat sample: SMEM on hash-partitioned rows while Chao1 is reliable and
 //    below 10^5 keys (any reliable Chao1 from 2^28 rows on); otherwise SORT (a
@@ -219,20 +226,17 @@ int64_t table_slots_from_sketch(const float* f, int64_t n) {
 //    rows from 2^25 rows on, SORT below.
 int rule_strategy(const float* f, uint32_t ops, double hll) {
   const KeyEstimate e = key_estimate(f);
-  const int cap = ops_minmax(ops) ? 1536 : 3072;  // 3/4 of the largest shared tables
+  const int cap = ops_minmax(ops) ? 1536 : 3072;  // 3/4 of the largest shared tables of every build
   const double coverage = 1.0 - (double)f[F_F1];  // F_F1 = f1 / m
   const float log2n = f[F_LOG2N];
   if (coverage >= 0.97) return AGG_STRAT_SMEM;
-  // with the column's HyperLogLog count: a hot head that shared tables absorb
-  // (the rest spilling to a right-sized table), or a flat column of up to 2^25
-  // keys (hash-partitioned shared tables); larger flat columns sort (on 2^30
-  // rows: 2^24 uniform keys 31 ms partitioned vs 43 ms sorted, 2^26 keys 59
-  // vs 45 ms)
   if (hll > 0.0) {
     if (hot_sample(f, cap) || hll <= cap) return AGG_STRAT_SMEM;
-    if (e.flat) return hll <= 33554432.0 ? AGG_STRAT_SMEM : AGG_STRAT_SORT;
+    if (log2n < 24.0f && hll > std::exp2((double)log2n) / 16.0) return AGG_STRAT_SORT;
+    return hll <= 33554432.0 || !e.flat ? AGG_STRAT_SMEM : AGG_STRAT_SORT;
   }
   if (log2n < 20.0f) return (e.plan <= cap || !e.flat) ? AGG_STRAT_SMEM : AGG_STRAT_GLOBAL;
+  if (!e.flat && coverage >= 0.7 && log2n < 22.0f) return AGG_STRAT_SMEM;
   const double m = std::min(std::exp2((double)log2n), (double)kSketchSample);
   const double d = (double)f[F_DISTINCT] * m, f1 = (double)f[F_F1] * m, f2 = (double)f[F_F2] * m;
   const double unseen = f1 * (f1 - 1.0) / (2.0 * (f2 + 1.0));  // Chao1's unseen keys
@@ -719,9 +723,13 @@ bool wants_hll(const float* f, int64_t n) {
   return n >= (int64_t(1) << 22) && 1.0 - (double)f[F_F1] < 0.97;
 }
 
+// A hot head that shared tables absorb: the sample covers 85% of the rows with
+// keys that fit a table; the rows of rarer keys go straight to the global table
+// (2^26 int32 rows, Zipf 1.3 over 10^6 keys: 0.98 ms, partitioned 1.49; at 73%
+// covered, 10^4 Zipf 1 keys, 1.22 ms, partitioned 0.88).
 bool hot_sample(const float* f, int cap) {
   const double m = std::min(std::exp2((double)f[F_LOG2N]), (double)kSketchSample);
-  return 1.0 - (double)f[F_F1] >= 0.9 && (double)f[F_DISTINCT] * m <= (double)cap;
+  return 1.0 - (double)f[F_F1] >= 0.85 && (double)f[F_DISTINCT] * m <= (double)cap;
 }
 
 // Global-table slots for a column with about `keys` distinct keys (a
@@ -761,7 +769,7 @@ static agg_status choose(const uint32_t* keys, const void* vals, int64_t n, int 
   c->plan.slots = tslots ? tslots
                          : hll > 0.0 ? slots_for_count(hll, n) : (have_feat ? table_slots_from_sketch(feat, n) : 2048);
   c->plan.smem_slots = sslots ? std::min(sslots, stab_max_slots(vdt, ops_minmax(ops), true))
-                              : smem_slots_for(est, ops_minmax(ops));
+                              : smem_slots_for(est, stab_max_slots(vdt, ops_minmax(ops), true));
   c->plan.threads_given = o.block_threads != 0;
   c->plan.smem_given = o.smem_slots != 0;
   c->plan.threads = o.block_threads ? o.block_threads : (strategy == AGG_STRAT_SMEM ? 512 : 256);
@@ -776,15 +784,16 @@ static agg_status choose(const uint32_t* keys, const void* vals, int64_t n, int 
   // half of L2; each partition then has about 1/256 of the keys.
   const double table_bytes = (double)(c->plan.slots + 2) * gslot_bytes(ops_minmax(ops));
   // a hot head that the shared tables absorb needs no partitioning: the few
-  // rows of rarer keys spill to the (right-sized) global table
-  const bool hot = hll > 0.0 && hot_sample(feat, (c->plan.smem_slots * 3) / 4);
+  // rows of rarer keys spill to the global table
+  const bool hot = have_feat && hot_sample(feat, (c->plan.smem_slots * 3) / 4);
   const bool spills = strategy == AGG_STRAT_SMEM && est > 0.75 * c->plan.smem_slots && !hot;
   const bool big_table = table_bytes > 0.5 * device_info().l2_bytes;
   c->plan.partition = o.partition > 0 || (o.partition == 0 && n >= (int64_t(1) << 20) && (spills || big_table));
   // two levels (65536 partitions) when 256 partitions would still spill
   c->plan.partition_passes =
       (o.partition == 2 ||
-       (o.partition == 0 && strategy == AGG_STRAT_SMEM && est > 256.0 * 0.75 * c->plan.smem_slots))
+       (o.partition == 0 && strategy == AGG_STRAT_SMEM &&
+        est > 256.0 * 0.75 * std::min(c->plan.smem_slots, stab_max_slots(vdt, ops_minmax(ops), false))))
           ? 2
           : 1;
   return AGG_OK;
