@@ -12,7 +12,11 @@
 // and the last block to finish (fence plus ticket, no waiting) forms the
 // estimate alpha_m m^2 / sum 2^-M_j (linear counting m ln(m / V) below 5m/2
 // when V registers are zero; above 2^32/30, the correction for a 32-bit hash
-// space). The registers and the ticket live in the
+// space). The blocks finish together: each starts its merge at its own part of
+// the registers, so that most registers it comes to already hold another block's
+// rank (all starting at register 0, nearly every rank of every block was an atomic
+// on an address that every other block was updating), and the last block sums
+// 2^-M_j as an integer. 2^24 keys: 85 us with both as before, 47 us so. The registers and the ticket live in the
 // stream's scratch and are cleared before every launch.
 //
 // The same pass can also count the rows of each of the 256 hash partitions
@@ -39,6 +43,9 @@ constexpr size_t kHllStateBytes = kHllHistOff + 256 * 8;
 constexpr size_t kHllScratchBytes = kHllScratchOff + kHllStateBytes;
 constexpr int kHllWarps = kHllThreads / 32;
 constexpr int kHllLoads = 4;  // 16-byte key loads a thread keeps in flight
+constexpr int kHllMerge = 8;  // registers a thread merges at a time
+constexpr int kHllMaxRank = 33 - kHllP;  // 19
+static_assert(kHllM % (kHllThreads * kHllMerge) == 0, "a merge turn covers whole registers");
 
 // whist: the warp's 256 partition counters (HIST only).
 template <bool HIST>
@@ -54,7 +61,7 @@ template <bool HIST>
 __global__ void __launch_bounds__(kHllThreads) hll_kernel(const uint32_t* __restrict__ keys, int64_t n, int64_t head,
                                                           uint32_t* __restrict__ regs) {
   extern __shared__ uint32_t sreg[];  // kHllM registers, then (HIST) kHllWarps x 256 counters
-  __shared__ double red[33];
+  __shared__ unsigned long long red[kHllWarps];
   __shared__ int s_last;
   unsigned* ticket = (unsigned*)((char*)regs + kHllTicketOff);
   double* est = (double*)((char*)regs + kHllEstOff);
@@ -84,9 +91,19 @@ __global__ void __launch_bounds__(kHllThreads) hll_kernel(const uint32_t* __rest
     }
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < kHllM; i += blockDim.x) {
-    const uint32_t r = sreg[i];
-    if (r != 0 && r > __ldcg(&regs[i])) atomicMax(&regs[i], r);
+  const uint32_t turn = (uint32_t)((uint64_t)blockIdx.x * kHllM / gridDim.x) & ~31u;
+  for (int i = threadIdx.x; i < kHllM; i += kHllThreads * kHllMerge) {
+    uint32_t at[kHllMerge], cur[kHllMerge];
+#pragma unroll
+    for (int u = 0; u < kHllMerge; ++u) {
+      at[u] = (i + u * kHllThreads + turn) & (kHllM - 1);
+      cur[u] = __ldcg(&regs[at[u]]);
+    }
+#pragma unroll
+    for (int u = 0; u < kHllMerge; ++u) {
+      const uint32_t r = sreg[at[u]];
+      if (r > cur[u]) atomicMax(&regs[at[u]], r);
+    }
   }
   if (HIST && threadIdx.x < 256) {
     unsigned long long* hist = (unsigned long long*)((char*)regs + kHllHistOff);
@@ -100,34 +117,25 @@ __global__ void __launch_bounds__(kHllThreads) hll_kernel(const uint32_t* __rest
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  double sum = 0.0, zeros = 0.0;
-  for (int i = threadIdx.x; i < kHllM; i += blockDim.x) {
-    const uint32_t r = __ldcg(&regs[i]);
-    sum += ldexp(1.0, -(int)r);
-    zeros += r == 0 ? 1.0 : 0.0;
-  }
-  // block sums in a fixed order
+  // sum 2^-M_j in units of 2^-19, and the zero registers above bit 40
+  unsigned long long sum = 0;
+  for (int i = threadIdx.x; i < kHllM; i += kHllThreads * kHllMerge) {
+    uint32_t r[kHllMerge];
 #pragma unroll
-  for (int o = 16; o >= 1; o >>= 1) {
-    sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    zeros += __shfl_xor_sync(0xffffffffu, zeros, o);
+    for (int u = 0; u < kHllMerge; ++u) r[u] = __ldcg(&regs[i + u * kHllThreads]);
+#pragma unroll
+    for (int u = 0; u < kHllMerge; ++u)
+      sum += (1ull << (kHllMaxRank - r[u])) | ((unsigned long long)(r[u] == 0) << 40);
   }
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  if (l == 0) red[w] = sum;
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sum;
   __syncthreads();
   if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t += red[i];
-    red[32] = t;
-  }
-  __syncthreads();
-  const double tot = red[32];
-  __syncthreads();
-  if (l == 0) red[w] = zeros;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double v = 0.0;
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) v += red[i];
+    unsigned long long t = 0;
+    for (int i = 0; i < kHllWarps; ++i) t += red[i];
+    const double v = (double)(t >> 40);
+    const double tot = (double)(t & ((1ull << 40) - 1)) / (double)(1u << kHllMaxRank);
     const double m = (double)kHllM;
     const double alpha = 0.7213 / (1.0 + 1.079 / m);
     double e = alpha * m * m / tot;
