@@ -205,11 +205,12 @@ int64_t table_slots_from_sketch(const float* f, int64_t n) {
 // int32 SUM/COUNT/MIN/MAX and float64 SUM/COUNT columns of 2^20 to 2^26 rows,
 // 3000 to 10^6 keys, uniform and Zipf 0.5 to 1.3; SMEM includes its partition):
 //  - the sample covers >= 97% of the mass: SMEM;
-//  - with the column's HyperLogLog count (2^22 rows and more): SMEM, from 2^24
-//    rows on (2^24 rows: 0.30-0.82 ms against 0.73-0.93 ms sorted) or while a
-//    key has 16 rows or more (below, the sort is up to 1.4x faster: 3 M rows
-//    over 950 K keys 0.32 ms against 0.44); flat columns of more than 2^25 keys
-//    sort (on 2^30 rows: 2^26 keys 45 ms sorted, 59 ms partitioned);
+//  - with the column's HyperLogLog count (2^22 rows and more): SMEM while a key
+//    has 16 rows or more, 12 from 2^24 rows on (float64, 24 M rows: 1.31 ms
+//    against 1.33 sorted at 16 rows a key, 2.00 against 1.34 at 8, 3.9 against
+//    1.6 at 2; 40 M rows: 1.89 against 2.05, 3.04 against 2.09, 6.1 against
+//    2.5; Zipf 1 keys cross at the same count); flat columns of more than 2^25
+//    keys sort (on 2^30 rows: 2^26 keys 45 ms sorted, 59 ms partitioned);
 //  - columns under 2^20 rows: SMEM for few keys or a skewed sample, else one
 //    global table;
 //  - a skewed sample covering 70% of a column under 2^22 rows: SMEM (3 M rows
@@ -232,7 +233,7 @@ int rule_strategy(const float* f, uint32_t ops, double hll) {
   if (coverage >= 0.97) return AGG_STRAT_SMEM;
   if (hll > 0.0) {
     if (hot_sample(f, cap) || hll <= cap) return AGG_STRAT_SMEM;
-    if (log2n < 24.0f && hll > std::exp2((double)log2n) / 16.0) return AGG_STRAT_SORT;
+    if (hll > std::exp2((double)log2n) / (log2n < 24.0f ? 16.0 : 12.0)) return AGG_STRAT_SORT;
     return hll <= 33554432.0 || !e.flat ? AGG_STRAT_SMEM : AGG_STRAT_SORT;
   }
   if (log2n < 20.0f) return (e.plan <= cap || !e.flat) ? AGG_STRAT_SMEM : AGG_STRAT_GLOBAL;
@@ -723,6 +724,20 @@ bool wants_hll(const float* f, int64_t n) {
   return n >= (int64_t(1) << 22) && 1.0 - (double)f[F_F1] < 0.97;
 }
 
+// A column that the rule sorts whatever its HyperLogLog count, which then is
+// not taken: so few repeats in the sample that it has more than about n^2 / 2.4e8
+// keys. (A sample of m rows repeats C(m, 2) sum p^2 >= m^2 / 2d times, so
+// frequent keys cannot hide.) Sorted without the count against partitioned with
+// it, float64: 4.2 M rows of 65 K keys 0.35 ms against 0.37; 9 M rows of 140 K
+// 0.55 against 0.47, of 560 K 0.56 against 0.61; 16 M rows of 250 K 0.86
+// against 0.64, of 1 M 0.88 against 0.89. From 2^25 rows on the sample no
+// longer tells such counts.
+bool sorts_uncounted(const float* f, int64_t n) {
+  if (n >= (int64_t(1) << 25)) return false;
+  const double repeats = (1.0 - (double)f[F_DISTINCT]) * (double)kSketchSample;
+  return repeats * (double)n * (double)n <= 2e15;
+}
+
 // A hot head that shared tables absorb: the sample covers 85% of the rows with
 // keys that fit a table; the rows of rarer keys go straight to the global table
 // (2^26 int32 rows, Zipf 1.3 over 10^6 keys: 0.98 ms, partitioned 1.49; at 73%
@@ -876,7 +891,7 @@ agg_status groupby_with(const uint32_t* keys, const void* vals, int64_t n, int v
       st = sketch_and_select(keys, n, vdt, ops, o.sample_offset, s, feat, &learned);
       if (st != AGG_OK) return st;
       have = true;
-      if (wants_hll(feat, n)) {
+      if (learned != AGG_STRAT_SORT && wants_hll(feat, n)) {
         st = hll_estimate(keys, n, s, &hll, part_counts);
         if (st != AGG_OK) return st;
         have_counts = true;
@@ -898,7 +913,7 @@ agg_status groupby_with(const uint32_t* keys, const void* vals, int64_t n, int v
     st = sketch_features(keys, n, vdt, ops, o.sample_offset, s, feat);
     if (st != AGG_OK) return st;
     have = true;
-    if (wants_hll(feat, n)) {
+    if (wants_hll(feat, n) && !(o.strategy == AGG_STRAT_AUTO && sorts_uncounted(feat, n))) {
       st = hll_estimate(keys, n, s, &hll, part_counts);
       if (st != AGG_OK) return st;
       have_counts = true;
