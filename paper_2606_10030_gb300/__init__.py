@@ -262,19 +262,28 @@ def check(status: int) -> None:
 
 
 def _stream_ptr(stream):
+    """The stream's handle as an int (null: 0); None is torch's current stream."""
+    if stream is not None:
+        return stream.cuda_stream
     import torch
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    if torch.cuda.is_initialized():  # without making a Stream object
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return torch.cuda.current_stream().cuda_stream
+
+
+_dtype_codes = None
 
 
 def dtype_code(t) -> int:
-    import torch
-    m = {torch.int32: AGG_I32, torch.int64: AGG_I64, torch.uint32: AGG_U32,
-         torch.float32: AGG_F32, torch.float64: AGG_F64}
-    if t.dtype not in m:
+    global _dtype_codes
+    if _dtype_codes is None:
+        import torch
+        _dtype_codes = {torch.int32: AGG_I32, torch.int64: AGG_I64, torch.uint32: AGG_U32,
+                        torch.float32: AGG_F32, torch.float64: AGG_F64}
+    code = _dtype_codes.get(t.dtype)
+    if code is None:
         raise TypeError(f"unsupported column dtype {t.dtype}")
-    return m[t.dtype]
+    return code
 
 
 def decode_scalar(buf) -> AggScalar:
@@ -294,13 +303,12 @@ def agg_reduce(col, ops: int = AGG_ALL, out=None, stream=None, n: int | None = N
     The result is written asynchronously on ``stream``; decode it with
     ``decode_scalar(out)`` (which synchronises by copying to the host).
     """
-    import torch
     assert col.is_cuda and col.dim() == 1 and col.is_contiguous()
     if out is None:
+        import torch
         out = torch.empty(SCALAR_BYTES, dtype=torch.uint8, device=col.device)
     n = col.numel() if n is None else n
-    check(lib().agg_reduce(ctypes.c_void_p(col.data_ptr()), n, dtype_code(col), ops,
-                           ctypes.c_void_p(out.data_ptr()), _stream_ptr(stream)))
+    check(lib().agg_reduce(col.data_ptr(), n, dtype_code(col), ops, out.data_ptr(), _stream_ptr(stream)))
     return out
 
 
@@ -354,12 +362,11 @@ def agg_pack_for(col) -> Packed:
 
 def agg_reduce_packed(p: Packed, ops: int = AGG_ALL, out=None, stream=None):
     """Ungrouped aggregation of a packed column held in device memory; returns the 80-byte device result."""
-    import torch
     assert p.buf.is_cuda
     if out is None:
+        import torch
         out = torch.empty(SCALAR_BYTES, dtype=torch.uint8, device=p.buf.device)
-    check(lib().agg_reduce_packed(ctypes.c_void_p(p.buf.data_ptr()), ctypes.byref(p.info), ops,
-                                  ctypes.c_void_p(out.data_ptr()), _stream_ptr(stream)))
+    check(lib().agg_reduce_packed(p.buf.data_ptr(), ctypes.byref(p.info), ops, out.data_ptr(), _stream_ptr(stream)))
     return out
 
 
@@ -385,16 +392,16 @@ class Groups:
 
     def __init__(self, ptr):
         self._ptr = ptr
-        g = ctypes.cast(ptr, ctypes.POINTER(AggGroups)).contents
-        self.num_groups = int(g.num_groups)
-        self.dtype = int(g.dtype)
-        self.ops = int(g.ops)
-        self.strategy = int(g.strategy)
-        self.retries = int(g.retries)
-        self.table_slots = int(g.table_slots)
-        self.smem_slots = int(g.smem_slots)
+        g = AggGroups.from_address(ptr)
+        self.num_groups = g.num_groups
+        self.dtype = g.dtype
+        self.ops = g.ops
+        self.strategy = g.strategy
+        self.retries = g.retries
+        self.table_slots = g.table_slots
+        self.smem_slots = g.smem_slots
         self.has_sum_err = bool(g.sum_err)
-        self.features = np.array(list(g.features), dtype=np.float32)
+        self.features = np.frombuffer(g.features, dtype=np.float32).copy()
 
     def to_host(self) -> dict:
         d = self.num_groups
@@ -440,9 +447,9 @@ def agg_groupby(keys, vals, ops: int = AGG_ALL, opts: AggOptions | None = None, 
     assert keys.is_contiguous() and vals.is_contiguous()
     n = keys.numel() if n is None else n
     out = ctypes.c_void_p()
-    check(lib().agg_groupby(ctypes.c_void_p(keys.data_ptr()), ctypes.c_void_p(vals.data_ptr()), n,
-                            dtype_code(vals), ops, ctypes.byref(opts) if opts is not None else None,
-                            ctypes.byref(out), _stream_ptr(stream)))
+    check(lib().agg_groupby(keys.data_ptr(), vals.data_ptr(), n, dtype_code(vals), ops,
+                            ctypes.byref(opts) if opts is not None else None, ctypes.byref(out),
+                            _stream_ptr(stream)))
     return Groups(out.value)
 
 
