@@ -412,13 +412,16 @@ agg_status radix_prepare() {
 //   part_scatter  per tile of 6144 or 8192 rows (a block of 512 threads, 12 or
 //                 16 rows a thread, the next tile's keys and values loaded
 //                 while the current one is written out): each row's place
-//                 among its warp's rows of the same digit from a per-warp
-//                 shared counter (a plain atomic: order within a partition is
-//                 free), the warps' counts scanned per digit, the tile's runs
-//                 reserved in the output with one global atomic per digit
-//                 (whose latency overlaps the scan and the staging), the
+//                 among the tile's rows of the same digit from a shared counter
+//                 (a plain atomic: order within a partition is free), the
+//                 tile's runs reserved in the output with one global atomic per
+//                 digit (whose latency overlaps the scan and the staging), the
 //                 rows staged in shared memory in digit order and written out
-//                 run by run.
+//                 run by run. One counter per digit and tile: with a set per
+//                 warp, merged per tile, every row also read its warp's offset
+//                 and the kernel was 8% slower (2^28 rows of 4-byte values in
+//                 two levels 2.85 ms, 2.60 now; 2^30 of 8-byte values 5.64 and
+//                 5.37 with the counts given, 4.8 TB/s).
 // Reads 4 + 12 B and writes 12 B per row (uint32 key, 8-byte value); no per-tile
 // count array and no ranking rounds. The histogram pass is skipped when the
 // caller already holds the counts (the GROUP BY planner's HyperLogLog pass
@@ -431,10 +434,11 @@ agg_status radix_prepare() {
 // ---------------------------------------------------------------------------
 constexpr int kPartHistThreads = 512;
 constexpr int kPartThreads = 512;
-// Rows per scatter tile and blocks per SM by payload: 8-byte values take
-// 8192-row tiles, one block a SM (112 KB of stage); 4-byte values 6144-row
-// tiles, two blocks a SM (longer runs per partition and fewer per-tile scans
-// than 4096-row tiles; measured on the 2^30-row partition: 5.6 vs 6.1 ms).
+// Rows per scatter tile and blocks per SM by payload (one level over 2^30 rows
+// of 8-byte values / two levels over 2^28 of 4-byte values): 8192 rows, one
+// block a SM 5.37 ms, 6144 rows, two blocks 5.43, one block of 1024 threads with
+// 8192 or 12288 rows 5.47 or 5.37; 4-byte values: 6144 rows, two blocks 2.60 ms,
+// 8192 (registers spill) 2.65, 1024 threads with 12288 or 16384 rows 2.74 or 2.80.
 template <class P>
 struct PartCfg {
   static constexpr int kTile = sizeof(P) == 8 ? 8192 : 6144;
@@ -588,12 +592,12 @@ __global__ void __launch_bounds__(kPartThreads, PartCfg<P>::kBlocks) part_scatte
                                                                 const unsigned long long* __restrict__ starts) {
   constexpr int kTile = PartCfg<P>::kTile;
   constexpr int kRows = kTile / kPartThreads;  // rows per thread and tile
-  constexpr int kWarps = kPartThreads / 32;
   extern __shared__ __align__(16) unsigned char sm_raw[];
   P* stage_v = (P*)sm_raw;                            // kTile
   uint32_t* stage_k = (uint32_t*)(stage_v + kTile);  // kTile
-  uint32_t* whist = stage_k + kTile;                 // kWarps x 256
+  __shared__ uint32_t hist[256];
   __shared__ uint32_t off[256];
+  __shared__ uint32_t wtot[8];
   __shared__ unsigned long long base[256];
   __shared__ int64_t first[SEG ? 257 : 1];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -638,66 +642,57 @@ __global__ void __launch_bounds__(kPartThreads, PartCfg<P>::kBlocks) part_scatte
     tile_of(t, r0, rows, fbase);
     load(r0, rows);
   }
-  for (int i = threadIdx.x; i < kWarps * 256; i += kPartThreads) whist[i] = 0;
+  if (threadIdx.x < 256) hist[threadIdx.x] = 0;
   __syncthreads();
   for (; t < ntiles; t += gridDim.x) {
-    uint32_t pr[kRows];
+    uint32_t dp[kRows];  // a row's digit, and above it its place among the tile's rows of that digit
 #pragma unroll
     for (int r = 0; r < kRows; ++r) {
       const int j = wbase + r * 32 + lane;
-      if (j < rows) pr[r] = atomicAdd(&whist[w * 256 + part_digit(kr[r], shift)], 1u);
+      const uint32_t d = part_digit(kr[r], shift);
+      if (j < rows) dp[r] = d | (atomicAdd(&hist[d], 1u) << 8);
     }
     __syncthreads();
-    // per digit: the warps' runs and the tile's count; the tile's run in the
-    // output is reserved now, its offset stored only after the staging (the
-    // atomic's latency overlaps the scan and the staging)
+    // the tile's run of every digit: its rows are reserved in the output now
+    // (the atomic's latency overlaps the scan and the staging), its place in the
+    // stage is the exclusive scan of the counts
     unsigned long long my_base = 0;
+    uint32_t run = 0, x = 0;
     if (threadIdx.x < 256) {
-      const int d = threadIdx.x;
-      uint32_t run = 0;
-      for (int ww = 0; ww < kWarps; ++ww) {
-        const uint32_t c = whist[ww * 256 + d];
-        whist[ww * 256 + d] = run;
-        run += c;
+      x = run = hist[threadIdx.x];
+      hist[threadIdx.x] = 0;  // for the next tile
+      if (run) my_base = atomicAdd(&fill[fbase + (int)threadIdx.x * kStride], (unsigned long long)run);
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
       }
-      off[d] = run;  // the tile's count of digit d, until the scan below
-      if (run) my_base = atomicAdd(&fill[fbase + d * kStride], (unsigned long long)run);
+      if (lane == 31) wtot[w] = x;
     }
     __syncthreads();
-    if (threadIdx.x < 32) {  // exclusive scan of the counts over digits
-      uint32_t run = 0;
-      for (int j = 0; j < 8; ++j) {
-        const uint32_t c = off[j * 32 + lane];
-        uint32_t x = c;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-          if (lane >= o) x += y;
-        }
-        off[j * 32 + lane] = run + x - c;
-        run += __shfl_sync(0xffffffffu, x, 31);
-      }
+    if (threadIdx.x < 256) {
+      x -= run;
+      for (int k = 0; k < w; ++k) x += wtot[k];
+      off[threadIdx.x] = x;
     }
     __syncthreads();
 #pragma unroll
     for (int r = 0; r < kRows; ++r) {
       const int j = wbase + r * 32 + lane;
       if (j < rows) {
-        const uint32_t d = part_digit(kr[r], shift);
-        const uint32_t p = off[d] + whist[w * 256 + d] + pr[r];
+        const uint32_t p = off[dp[r] & 255u] + (dp[r] >> 8);
         stage_k[p] = kr[r];
         stage_v[p] = vr[r];
       }
     }
     // a row at stage position p goes to base[d] + p (mod 2^64)
-    if (threadIdx.x < 256) base[threadIdx.x] = my_base - (unsigned long long)off[threadIdx.x];
+    if (threadIdx.x < 256) base[threadIdx.x] = my_base - (unsigned long long)x;
     const int rows_now = rows;
     if (t + gridDim.x < ntiles) {
       tile_of(t + gridDim.x, r0, rows, fbase);
       load(r0, rows);
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < kWarps * 256; i += kPartThreads) whist[i] = 0;  // for the next tile
     for (int p = threadIdx.x; p < rows_now; p += kPartThreads) {
       const uint32_t key = stage_k[p];
       const uint32_t d = part_digit(key, shift);
@@ -772,7 +767,7 @@ __global__ void __launch_bounds__(256) seg_starts(unsigned long long* __restrict
 
 template <class P>
 static size_t part_smem() {
-  return (size_t)PartCfg<P>::kTile * (sizeof(P) + 4) + (size_t)(kPartThreads / 32) * 256 * 4;
+  return (size_t)PartCfg<P>::kTile * (sizeof(P) + 4);
 }
 
 size_t partition_tmp_bytes() { return (257 * kFillStride) * sizeof(unsigned long long) + 256; }
