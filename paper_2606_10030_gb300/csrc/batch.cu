@@ -538,7 +538,7 @@ static agg_status plan_enqueue(agg_batch_plan* P, cudaStream_t s, int64_t* kerne
                                                (uint64_t*)P->cp, L, (const int64_t*)P->ccount, 32, P->rtmp, s, &kout,
                                                &pout);
     if (st != AGG_OK) return st;
-    k += 4 * 5;
+    k += 4 * 3;
     // stage 2: stably by query id (16 bits), (key, slot) as the payload
     uint32_t* k2 = kout == P->ck ? P->ck2 : P->ck;
     uint64_t* p2 = pout == (uint64_t*)P->cp ? (uint64_t*)P->cp2 : (uint64_t*)P->cp;
@@ -550,7 +550,7 @@ static agg_status plan_enqueue(agg_batch_plan* P, cudaStream_t s, int64_t* kerne
     st = radix_sort_pairs<uint64_t>(k2, p2, kout, pout, k2, p2, L, (const int64_t*)P->ccount, 16, P->rtmp, s, &kfin,
                                     &pfin);
     if (st != AGG_OK) return st;
-    k += 2 * 5;
+    k += 2 * 3;
     batch_first<<<1, 32, 0, s>>>(P->dq, P->nq, P->is_large, P->first);
     batch_gather<<<(unsigned)g, 256, 0, s>>>(P->dq, kfin, (const unsigned long long*)pfin, P->ccount, P->first, L);
     k += 2;

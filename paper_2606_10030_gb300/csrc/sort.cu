@@ -109,32 +109,28 @@ size_t scan_tmp_bytes(int64_t n) {
   return (size_t)(nb > 0 ? nb : 1) * sizeof(uint32_t) + 256;
 }
 
-// Up to kScanSmall values: one block, in place of three launches (11 us for
-// 6000 values, 5 us here).
-constexpr int64_t kScanSmall = int64_t(1) << 16;
+// Up to kScanSmall values: one turn of one block, in place of three launches (11
+// us for 6000 values, 5 us here; every further turn is another 6 us).
 constexpr int kScanSmallThreads = 1024;
+constexpr int64_t kScanSmall = 8 * kScanSmallThreads;
 __global__ void __launch_bounds__(kScanSmallThreads) scan_small(const uint32_t* in, uint32_t* out, int n,
                                                                 uint32_t* total) {
-  uint32_t carry = 0;
-  for (int b = 0; b < n; b += kScanSmallThreads * 8) {
-    const int j = b + (int)threadIdx.x * 8;
-    uint32_t v[8];
-    uint32_t sum = 0;
+  const int j = (int)threadIdx.x * 8;
+  uint32_t v[8];
+  uint32_t sum = 0;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      v[i] = j + i < n ? in[j + i] : 0u;
-      sum += v[i];
-    }
-    uint32_t all;
-    uint32_t e = carry + block_exclusive_scan(sum, &all);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      if (j + i < n) out[j + i] = e;
-      e += v[i];
-    }
-    carry += all;
+  for (int i = 0; i < 8; ++i) {
+    v[i] = j + i < n ? in[j + i] : 0u;
+    sum += v[i];
   }
-  if (threadIdx.x == 0 && total) *total = carry;
+  uint32_t all;
+  uint32_t e = block_exclusive_scan(sum, &all);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    if (j + i < n) out[j + i] = e;
+    e += v[i];
+  }
+  if (threadIdx.x == 0 && total) *total = all;
 }
 
 agg_status scan_exclusive_u32(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* total_dev, void* tmp,
@@ -241,11 +237,17 @@ __global__ void __launch_bounds__(kRowsThreads) radix_rows(uint32_t* __restrict_
 // 1. each warp ranks its rows among equal digits, round by round, with
 //    digit-bit ballots and a per-warp running digit count (ranks stay in
 //    registers);
-// 2. digit totals are scanned across warps and digits, and the tile's digit
-//    starts folded into the per-warp offsets and the global offsets;
+// 2. digit counts are summed over warps and scanned over digits together with
+//    the column's digit totals, and every warp's rows get their place;
 // 3. values are loaded (keys are in registers) and rows staged in shared
 //    memory in digit order;
 // 4. each digit's run is written to its global offset with coalesced stores.
+// Bound by instruction issue and barriers in turn (half of the issue slots). 16 M
+// rows of 8-byte values: 110 us a pass, 3.5 TB/s (133 us with two scans, six
+// barriers, in step 2, ranks of a register each and two rounds over the warps'
+// counts; with the values copied to the stage by cp.async during step 1, 155 us:
+// they cost the registers that hold three blocks on an SM). 2 M rows of 4-byte
+// values: 22.2 -> 19.5 us.
 template <class P>
 __global__ void __launch_bounds__(kSortThreads, 3) radix_scatter(const uint32_t* __restrict__ keys,
                                                               const P* __restrict__ vals, uint32_t* __restrict__ okeys,
@@ -260,6 +262,7 @@ __global__ void __launch_bounds__(kSortThreads, 3) radix_scatter(const uint32_t*
   uint32_t* whist = stage_k + kSortTile;                 // kWarps x 256
   uint32_t* gbase = whist + kWarps * 256;                // 256
 
+  __shared__ unsigned long long wsum[8];
   const int64_t n = rows_of(n_cap, n_dev);
   const int64_t tile0 = (int64_t)blockIdx.x * kSortTile;
   if (tile0 >= n) return;
@@ -267,7 +270,8 @@ __global__ void __launch_bounds__(kSortThreads, 3) radix_scatter(const uint32_t*
   for (int i = threadIdx.x; i < kWarps * 256; i += kSortThreads) whist[i] = 0;
   __syncthreads();
 
-  uint32_t lr[kSortItems];
+  static_assert(kSortItems == 8, "a warp ranks 256 rows, so ranks are bytes");
+  uint32_t lr[2] = {0, 0};  // ranks, a byte each
   uint32_t kr[kSortItems];
   const uint32_t lt = (1u << lane) - 1u;
   const int64_t wbase = tile0 + (int64_t)w * (kSortItems * 32);
@@ -290,34 +294,47 @@ __global__ void __launch_bounds__(kSortThreads, 3) radix_scatter(const uint32_t*
       peers &= bit ? m : ~m;
     }
     const uint32_t before = ok ? whist[w * 256 + d] : 0u;
-    lr[r] = before + __popc(peers & lt);
+    const uint32_t rank = before + __popc(peers & lt);
+    lr[r / 4] |= rank << (8 * (r % 4));
     __syncwarp();
     if (ok && (peers & lt) == 0) whist[w * 256 + d] = before + __popc(peers);
     __syncwarp();
   }
+  uint32_t tot = 0, before_tile = 0;  // of this thread's digit: rows of the column, rows in earlier tiles
+  if (threadIdx.x < 256) {
+    tot = totals[threadIdx.x];
+    before_tile = offsets[(int64_t)threadIdx.x * stride + blockIdx.x];
+  }
   __syncthreads();
-  {  // per digit: exclusive prefix over warps, then over digits
-    uint32_t run = 0;
-    if (threadIdx.x < 256) {
-      const int d = threadIdx.x;
+  // Per digit: the tile's count over its warps, and one scan over the digits of
+  // that count (high word: the digit's place in the stage) and the digit's rows
+  // in the whole column (low word: its place in the output).
+  const bool dig = threadIdx.x < 256;
+  uint32_t run = 0;
+  unsigned long long own = 0, x = 0;
+  if (dig) {
 #pragma unroll
-      for (int ww = 0; ww < kWarps; ++ww) {
-        const uint32_t c = whist[ww * 256 + d];
-        whist[ww * 256 + d] = run;
-        run += c;
-      }
+    for (int ww = 0; ww < kWarps; ++ww) run += whist[ww * 256 + threadIdx.x];
+    x = own = ((unsigned long long)run << 32) | tot;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
     }
-    const uint32_t e = block_exclusive_scan(threadIdx.x < 256 ? run : 0u, nullptr);
-    // the digit's global offset: the lower digits' rows, and its rows in earlier tiles
-    uint32_t goff = block_exclusive_scan(threadIdx.x < 256 ? totals[threadIdx.x] : 0u, nullptr);
-    if (threadIdx.x < 256) {
-      goff += offsets[(int64_t)threadIdx.x * stride + blockIdx.x];
-      // fold the digit's tile start into its per-warp offsets, and its global
-      // offset minus the tile start into gbase (mod 2^32: positions are < 2^32)
-      const int d = threadIdx.x;
+    if (lane == 31) wsum[w] = x;
+  }
+  __syncthreads();
+  if (dig) {
+    x -= own;
+    for (int k = 0; k < w; ++k) x += wsum[k];
+    uint32_t at = (uint32_t)(x >> 32);
+    // its global offset minus its place in the stage (mod 2^32: positions are < 2^32)
+    gbase[threadIdx.x] = (uint32_t)x + before_tile - at;
 #pragma unroll
-      for (int ww = 0; ww < kWarps; ++ww) whist[ww * 256 + d] += e;
-      gbase[d] = goff - e;
+    for (int ww = 0; ww < kWarps; ++ww) {  // the places of its warps' rows
+      const uint32_t c = whist[ww * 256 + threadIdx.x];
+      whist[ww * 256 + threadIdx.x] = at;
+      at += c;
     }
   }
   __syncthreads();
@@ -327,7 +344,7 @@ __global__ void __launch_bounds__(kSortThreads, 3) radix_scatter(const uint32_t*
     if (j < n) {
       const uint32_t key = kr[r];
       const uint32_t d = digit_of(key, shift, kbase);
-      const uint32_t lp = whist[w * 256 + d] + lr[r];
+      const uint32_t lp = whist[w * 256 + d] + ((lr[r / 4] >> (8 * (r % 4))) & 255u);
       stage_k[lp] = key;
       stage_v[lp] = vals[j];
     }
