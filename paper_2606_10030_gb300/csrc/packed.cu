@@ -8,14 +8,17 @@
 // link (agg_reduce_packed_host) or are read from HBM (agg_reduce_packed).
 //
 // Decode: a warp takes a frame; lane l holds values l, l + 32, ..., so the
-// 32 lanes of one step read one contiguous span of 32 * bits bits (the words
-// they share come from L1), and a lane's bit offset within its word is the same
+// 32 lanes of one step read one contiguous span of 32 * bits bits (words they
+// share are one access), and a lane's bit offset within its word is the same
 // in every step: of up to 32 bits a value is one funnel shift of two words and
 // a mask. The steps sum, minimise and maximise the packed offsets; the frame's
-// reference is added once. 2^25 int32 rows of 17 bits: 86 us when every value
-// computed its own 64-bit position and was folded as a whole value, 33
-// us now, at 2.1 TB/s bound by the latency of the word loads (half of the issue
-// slots are used, 9 of 16 cycles between a warp's instructions wait for loads).
+// reference is added once. A frame's words come through shared memory: while a
+// warp folds one frame, the next is copied there (three blocks of eight warps, two
+// frames a warp, keep 50 KB in flight an SM). 2^25 int32 rows of 17 bits, from
+// HBM: 104 us a call when every value computed its own 64-bit position and was
+// folded as a whole value and a second launch merged, 40.6 us with the words
+// loaded where they are used, 30.9 us now (2.3 TB/s), bound by the instructions of
+// the extraction (19 a warp and 32 values) and the latency of its shared loads.
 #include <algorithm>
 #include <cstring>
 #include <map>
@@ -53,6 +56,25 @@ __device__ __forceinline__ typename Traits<DT>::T unpack_value(const uint32_t* _
   return (T)(ref + (int64_t)x);
 }
 
+// A warp's stage: two frames of up to 32 bits a value, and the look-ahead word
+// (its value does not matter: the mask drops it).
+constexpr int kStageWords = AGG_PACK_FRAME + 4;
+constexpr int kPackBlocksPerSm = 3;
+constexpr size_t kPackSmem = (size_t)(kBlock / 32) * 2 * kStageWords * 4;
+
+__device__ __forceinline__ bool stageable(const PackDesc& d, const uint32_t* w) {
+  return d.bits - 1u < 32u && ((uintptr_t)w & 15) == 0;
+}
+
+// Start copying the words of the frame's first cnt values.
+__device__ __forceinline__ void stage_frame(uint32_t* stage, const uint32_t* __restrict__ w, uint32_t bits, int cnt,
+                                            int lane) {
+  const int quads = (int)(((uint32_t)cnt * bits + 127) / 128);  // at most the frame's 8 * bits
+  const uint32_t dst = (uint32_t)__cvta_generic_to_shared(stage);
+  for (int c = lane; c < quads; c += 32)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16 * c), "l"(w + 4 * c));
+}
+
 // A frame of up to 32 bits a value: the sum, minimum and maximum of this
 // lane's packed offsets among the first cnt values.
 template <bool SUM, bool MM>
@@ -67,8 +89,8 @@ __device__ __forceinline__ void fold_narrow(const uint32_t* __restrict__ w, uint
 #pragma unroll
     for (int u = 0; u < kSteps; ++u) {
       const bool in = i + 32 * u < cnt;
-      lo[u] = in ? __ldg(p + u * bits) : 0u;
-      hi[u] = in ? __ldg(p + u * bits + 1) : 0u;
+      lo[u] = in ? p[u * bits] : 0u;
+      hi[u] = in ? p[u * bits + 1] : 0u;
     }
 #pragma unroll
     for (int u = 0; u < kSteps; ++u) {
@@ -87,7 +109,7 @@ __device__ __forceinline__ void fold_narrow(const uint32_t* __restrict__ w, uint
 // buffer (word offsets counted from words_base). ticket: the last block merges
 // the partials into *out (null: another launch does).
 template <int DT, bool SUM, bool MM>
-__global__ void __launch_bounds__(kBlock) packed_scan(const PackDesc* __restrict__ desc, const uint32_t* __restrict__ words,
+__global__ void __launch_bounds__(kBlock, kPackBlocksPerSm) packed_scan(const PackDesc* __restrict__ desc, const uint32_t* __restrict__ words,
                                                       uint64_t words_base, int64_t f0, int64_t nf, int64_t n,
                                                       Partial* __restrict__ parts, int part_base, unsigned* ticket,
                                                       agg_scalar* out, uint32_t ops) {
@@ -97,19 +119,36 @@ __global__ void __launch_bounds__(kBlock) packed_scan(const PackDesc* __restrict
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * kBlock + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * kBlock) >> 5;
-  PackDesc d{};
-  if (warp < nf) d = desc[warp];
+  extern __shared__ __align__(16) uint32_t pack_smem[];
+  uint32_t* stage = pack_smem + (threadIdx.x >> 5) * (2 * kStageWords);
+  auto words_of = [&](const PackDesc& x) { return words + (x.word_off - words_base); };
+  auto values_of = [&](int64_t f) { return (int)min((int64_t)AGG_PACK_FRAME, n - (f0 + f) * AGG_PACK_FRAME); };
+  // while a frame is folded, the next one's words and the descriptor after it are in flight
+  PackDesc d{}, next{};
+  if (warp < nf) {
+    d = desc[warp];
+    if (stageable(d, words_of(d))) stage_frame(stage, words_of(d), d.bits, values_of(warp), lane);
+  }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  if (warp + nwarps < nf) next = desc[warp + nwarps];
+  uint32_t* now = stage;
+  uint32_t* then = stage + kStageWords;
   for (int64_t f = warp; f < nf; f += nwarps) {
-    PackDesc next{};
-    if (f + nwarps < nf) next = desc[f + nwarps];  // in flight while this frame is folded
-    const uint32_t* w = words + (d.word_off - words_base);
-    const int64_t row0 = (f0 + f) * AGG_PACK_FRAME;
-    const int cnt = (int)min((int64_t)AGG_PACK_FRAME, n - row0);
+    if (f + nwarps < nf && stageable(next, words_of(next)))
+      stage_frame(then, words_of(next), next.bits, values_of(f + nwarps), lane);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    PackDesc after{};
+    if (f + 2 * nwarps < nf) after = desc[f + 2 * nwarps];
+    const uint32_t* w = words_of(d);
+    const int cnt = values_of(f);
     const int mine = cnt > lane ? (cnt - lane + 31) / 32 : 0;  // this lane's values
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncwarp();
     if (d.bits <= 32) {
       uint64_t sum = 0;
       uint32_t mn = 0xFFFFFFFFu, mx = 0;
       if (d.bits == 0) mn = 0;
+      else if (stageable(d, w)) fold_narrow<SUM, MM>(now, d.bits, cnt, lane, sum, mn, mx);
       else fold_narrow<SUM, MM>(w, d.bits, cnt, lane, sum, mn, mx);
       if (SUM) a.s += (int64_t)(sum + (uint64_t)mine * (uint64_t)d.ref);
       if (MM && mine) {
@@ -121,7 +160,13 @@ __global__ void __launch_bounds__(kBlock) packed_scan(const PackDesc* __restrict
       for (int i = lane; i < cnt; i += 32) a.fold(unpack_value<DT>(w, d.bits, d.ref, i));
     }
     d = next;
+    next = after;
+    __syncwarp();  // every lane is done with the stage before it is filled again
+    uint32_t* const t = now;
+    now = then;
+    then = t;
   }
+  asm volatile("cp.async.wait_all;" ::: "memory");
   Partial p;
   a.to_partial(p, 0);
   p = block_reduce<Traits<DT>::FP, kBlock>(p);
@@ -172,7 +217,7 @@ static void* pick_packed_merge(int dt) {
 static int packed_grid(int64_t nf) {
   const DeviceInfo& di = device_info();
   const int64_t warps_per_block = kBlock / 32;
-  int64_t g = (int64_t)di.sm_count * 8;
+  int64_t g = (int64_t)di.sm_count * kPackBlocksPerSm;
   const int64_t need = (nf + warps_per_block - 1) / warps_per_block;
   if (need < g) g = need;
   return (int)std::max<int64_t>(1, g);
@@ -295,7 +340,9 @@ extern "C" agg_status agg_reduce_packed(const void* packed_dev, const agg_packed
     unsigned* ticket = (unsigned*)scratch;  // zero between calls: the last block leaves it so
     void* args[] = {(void*)&desc, (void*)&words, (void*)&base, (void*)&f0, (void*)&nf, (void*)&n, (void*)&parts,
                     (void*)&part_base, (void*)&ticket, (void*)&out_dev, (void*)&ops};
-    AGG_CUDA_TRY(cudaLaunchKernel(pick_packed(info->dtype, sum, mm), dim3(grid), dim3(kBlock), args, 0, s));
+    void* fn = pick_packed(info->dtype, sum, mm);
+    AGG_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPackSmem));
+    AGG_CUDA_TRY(cudaLaunchKernel(fn, dim3(grid), dim3(kBlock), args, kPackSmem, s));
     note_launch();
   }
   return AGG_OK;
@@ -373,6 +420,7 @@ extern "C" agg_status agg_reduce_packed_host(const void* packed_host, const agg_
   cudaStreamWaitEvent(pipe->copy, start_ev, 0);
   const bool sum = ops & (AGG_SUM | AGG_AVG), mm = ops & (AGG_MIN | AGG_MAX);
   void* fn = pick_packed(info->dtype, sum, mm);
+  AGG_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPackSmem));
   int64_t n = info->n;
   const int64_t total_words = info->nwords;
   for (int64_t c = 0; c < nchunks; ++c) {
@@ -397,7 +445,7 @@ extern "C" agg_status agg_reduce_packed_host(const void* packed_host, const agg_
     agg_scalar* no_out = nullptr;
     void* args[] = {(void*)&dd, (void*)&wd, (void*)&base, (void*)&ff0, (void*)&nff, (void*)&n, (void*)&parts,
                     (void*)&part_base, (void*)&no_ticket, (void*)&no_out, (void*)&ops};
-    AGG_CUDA_TRY(cudaLaunchKernel(fn, dim3(grid), dim3(kBlock), args, 0, s));
+    AGG_CUDA_TRY(cudaLaunchKernel(fn, dim3(grid), dim3(kBlock), args, kPackSmem, s));
     note_launch();
     cudaEventRecord(pipe->freed[b], s);
   }
