@@ -64,3 +64,25 @@ def test_sort_of_more_tiles_than_one_turn_of_the_digit_scan():
     keys = keyed_rows(n, 50_000, 10)
     vals = dg.values("i32", n, 11)
     check_groups(run(keys, vals, agg.AGG_STRAT_SORT)[0], keys, vals, agg.AGG_ALL)
+
+
+@pytest.mark.parametrize("distinct,skew,strategy", [(1 << 20, 0.0, "SORT"), (4000, 0.0, "SMEM"), (20_000, 1.0, "SMEM")])
+def test_auto_around_the_distinct_count(distinct, skew, strategy):
+    """Columns that AUTO sorts without a distinct count, and that it builds in tables with one."""
+    n = (1 << 22) + 5
+    keys = dg.keys_zipf(n, distinct, skew, 12) if skew else keyed_rows(n, distinct, 12)
+    vals = dg.values("f64", n, 13)
+    res, (used, _, _) = run(keys, vals, agg.AGG_STRAT_AUTO)
+    assert used == getattr(agg, "AGG_STRAT_" + strategy)
+    check_groups(res, keys, vals, agg.AGG_ALL)
+
+
+def test_runs_across_chunks_and_lanes():
+    """Sorted runs of every length around a lane's 8 rows and a warp's 256, alone and in sequence."""
+    lengths = np.concatenate([np.arange(1, 40), [255, 256, 257, 511, 512, 513, 2047, 2049], np.ones(300, int),
+                              np.full(60, 8), [5000]]).astype(np.int64)
+    keys = np.repeat(np.arange(lengths.size, dtype=np.uint32) * 7 + 3, lengths)
+    for dt in ("i64", "f32", "f64", "u32"):
+        vals = dg.values(dt, keys.size, 14)
+        for ops in (agg.AGG_ALL, agg.AGG_SUM | agg.AGG_COUNT):
+            check_groups(run(keys, vals, agg.AGG_STRAT_SORT, ops)[0], keys, vals, ops)
