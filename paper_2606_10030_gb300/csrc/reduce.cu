@@ -22,7 +22,10 @@
 // converts the total to float64 at the end. The order is fixed, so the result
 // is deterministic for a given grid. Measured against float64 TwoSum merges in
 // every shuffle step: 2^20 int32 rows 17.7 -> 8.7 us a call, 10^8 float64
-// rows 207 -> 178 us (with the scale started from the warp's first rows).
+// rows 207 -> 178 us (with the scale started from the warp's first rows), 167 us
+// with two rows sharing the fast-path and MIN/MAX tests (SUM alone 131 -> 125;
+// bound by integer issue: five blocks a SM with 48 registers, no spill, take the
+// same 167 us).
 //
 // Error bound of a float SUM. It adds up the roundings that can occur: per
 // thread, those of the compensation word of a float32 pair (each at most 2^-24
@@ -68,19 +71,15 @@ __global__ void __launch_bounds__(kBlock, DT == AGG_I64 && MM ? 4 : 6) reduce_sc
       a.fx.start(__reduce_max_sync(0xffffffffu, max((r.y >> 20) & 0x7FFu, (r.w >> 20) & 0x7FFu)));
     }
     for (int64_t base = (int64_t)blockIdx.x * kBlock * kUnroll + threadIdx.x; base < nv; base += stride) {
+      const int left = (int)min(nv - base, (int64_t)kUnroll * kBlock);  // vector u exists when u * kBlock < left
       uint4 r[kUnroll];
 #pragma unroll
-      for (int u = 0; u < kUnroll; ++u) {
-        const int64_t i = base + (int64_t)u * kBlock;
-        r[u] = i < nv ? ld_stream_v4(v + i) : make_uint4(0, 0, 0, 0);
-      }
+      for (int u = 0; u < kUnroll; ++u)
+        r[u] = u * kBlock < left ? ld_stream_v4(v + base + u * kBlock) : make_uint4(0, 0, 0, 0);
 #pragma unroll
-      for (int u = 0; u < kUnroll; ++u) {
-        if (base + (int64_t)u * kBlock < nv) {
-          a.fold_vec(r[u]);
-          rows += EPV;
-        }
-      }
+      for (int u = 0; u < kUnroll; ++u)
+        if (u * kBlock < left) a.fold_vec(r[u]);
+      rows += EPV * (uint32_t)((left + kBlock - 1) / kBlock);
     }
   }
   Partial p;

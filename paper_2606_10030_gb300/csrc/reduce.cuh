@@ -98,20 +98,24 @@ template <> struct FpImg<double> {
 // on the side, so that a column holding one sums to a non-finite value.
 // GB300 issues few float64 operations per clock (a TwoSum per row held the
 // float64 scan to 0.6 TB/s); this takes only integer operations per row.
+// E starts at kFixFirst, where the unit is the smallest subnormal: nothing is
+// lost there, and the exponent field of a subnormal (0) lies below every base,
+// so that one test on the high word selects the fast path.
 constexpr int kFixGuard = 31;
+constexpr int kFixFirst = kFixGuard + 1;
 
 struct Fix128 {
   uint64_t lo, hi;
   uint32_t nneg;  // negative rows added on the fast path as ~v, each still owing +1
   int E;
-  int base;       // E - kFixGuard: a row of exponent field e sits e - base bits up
+  uint32_t base;  // (E - kFixGuard) << 20: a row's high word minus this holds the row's shift
   uint32_t special;  // kPosInf | kNegInf | kNan
   __device__ void init() {
     lo = 0;
     hi = 0;
     nneg = 0;
-    E = 0;
-    base = -kFixGuard;
+    E = kFixFirst;
+    base = 1u << 20;
     special = 0;
   }
   // Scale for rows of exponent fields up to ef + 1 (the sum so far is zero or exact).
@@ -141,38 +145,49 @@ struct Fix128 {
     fold_neg();
     shift_right(lo, hi, e - E);
     E = e;
-    base = e - kFixGuard;
+    base = (uint32_t)(e - kFixGuard) << 20;
+  }
+  // A row's high word relative to base. Bits 20 to 30 hold ef - (E - kFixGuard)
+  // mod 2^11 (1 <= E - kFixGuard <= 2015): the shift, 0 to 31, of a normal value
+  // within kFixGuard binades of E, and 32 or more (a bit of kFixOut is set) for
+  // every other row.
+  static constexpr uint32_t kFixOut = 0x7E000000u;
+  __device__ __forceinline__ uint32_t rel(uint32_t uh) const { return uh - base; }
+  // A row on the fast path (x = rel(uh)): its 53-bit significand m, in one's
+  // complement when negative (the +1 counted in nneg), shifted left by less
+  // than 32 on 32-bit words (three funnel shifts, which use the low five bits of
+  // the amount), added with one carry chain.
+  __device__ __forceinline__ void add_fast(uint32_t uh, uint32_t ul, uint32_t x) {
+    static_assert(kFixGuard == 31, "the fast path shifts by less than one word");
+    const unsigned sh = x >> 20;
+    const uint32_t s = (uint32_t)((int32_t)uh >> 31);            // all ones for a negative row
+    const uint32_t mh = ((uh & 0x000FFFFFu) | 0x00100000u) ^ s;  // m's high 21 bits (implicit bit included)
+    const uint32_t ml = ul ^ s;
+    const uint32_t x0 = __funnelshift_l(s, ml, sh);
+    const uint32_t x1 = __funnelshift_l(ml, mh, sh);
+    const uint32_t x2 = __funnelshift_l(mh, s, sh);  // m >> (32 - sh), 0 when sh = 0
+    const uint32_t x3 = s;
+    asm("{\n\t.reg .u32 a0, a1, a2, a3;\n\t"
+        "mov.b64 {a0, a1}, %0;\n\t"
+        "mov.b64 {a2, a3}, %1;\n\t"
+        "add.cc.u32 a0, a0, %2;\n\t"
+        "addc.cc.u32 a1, a1, %3;\n\t"
+        "addc.cc.u32 a2, a2, %4;\n\t"
+        "addc.u32 a3, a3, %5;\n\t"
+        "mov.b64 %0, {a0, a1};\n\t"
+        "mov.b64 %1, {a2, a3};\n\t}"
+        : "+l"(lo), "+l"(hi)
+        : "r"(x0), "r"(x1), "r"(x2), "r"(x3));
+    nneg -= s;
   }
   __device__ __forceinline__ void add(uint64_t u) {
     const uint32_t uh = (uint32_t)(u >> 32), ul = (uint32_t)u;
-    const int ef = (int)((uh >> 20) & 0x7FFu);
-    const int sh = ef - base;  // E - ef binades below E: sh = kFixGuard - (E - ef)
-    if ((unsigned)sh <= (unsigned)kFixGuard && ef != 0) {
-      // fast path: a normal value within kFixGuard binades of E. Its 53-bit
-      // significand m shifted left by sh (< 32) on 32-bit words (three funnel
-      // shifts), in one's complement when negative (the +1 counted in nneg),
-      // added with one carry chain.
-      static_assert(kFixGuard < 32, "the fast path shifts by less than one word");
-      const uint32_t mh = (uh & 0x000FFFFFu) | 0x00100000u;  // m's high 21 bits (implicit bit included)
-      const uint32_t s = (uint32_t)((int32_t)uh >> 31);      // all ones for a negative row
-      const uint32_t x0 = __funnelshift_l(0u, ul, (unsigned)sh) ^ s;
-      const uint32_t x1 = __funnelshift_l(ul, mh, (unsigned)sh) ^ s;
-      const uint32_t x2 = __funnelshift_l(mh, 0u, (unsigned)sh) ^ s;  // m >> (32 - sh), 0 when sh = 0
-      const uint32_t x3 = s;
-      asm("{\n\t.reg .u32 a0, a1, a2, a3;\n\t"
-          "mov.b64 {a0, a1}, %0;\n\t"
-          "mov.b64 {a2, a3}, %1;\n\t"
-          "add.cc.u32 a0, a0, %2;\n\t"
-          "addc.cc.u32 a1, a1, %3;\n\t"
-          "addc.cc.u32 a2, a2, %4;\n\t"
-          "addc.u32 a3, a3, %5;\n\t"
-          "mov.b64 %0, {a0, a1};\n\t"
-          "mov.b64 %1, {a2, a3};\n\t}"
-          : "+l"(lo), "+l"(hi)
-          : "r"(x0), "r"(x1), "r"(x2), "r"(x3));
-      nneg -= s;
+    const uint32_t x = rel(uh);
+    if ((x & kFixOut) == 0u) {
+      add_fast(uh, ul, x);
       return;
     }
+    const int ef = (int)((uh >> 20) & 0x7FFu);
     fold_neg();
     if (ef == 0x7FF) {  // infinity or NaN
       special |= (u & 0x000FFFFFFFFFFFFFull) ? kNan : (int64_t)u < 0 ? kNegInf : kPosInf;
@@ -276,8 +291,27 @@ struct Acc<DT, SUM, MM, true> {
       fold(__uint_as_float(r.x)); fold(__uint_as_float(r.y));
       fold(__uint_as_float(r.z)); fold(__uint_as_float(r.w));
     } else {
-      fold(__longlong_as_double((long long)(((uint64_t)r.y << 32) | r.x)));
-      fold(__longlong_as_double((long long)(((uint64_t)r.w << 32) | r.z)));
+      // two rows share the tests for the fixed-point sum's fast path and for a
+      // high word that may move an extreme
+      if (SUM) {
+        const uint32_t x0 = fx.rel(r.y), x1 = fx.rel(r.w);
+        if (((x0 | x1) & Fix128::kFixOut) == 0u) {
+          fx.add_fast(r.y, r.x, x0);
+          fx.add_fast(r.w, r.z, x1);
+        } else {
+          fx.add(((uint64_t)r.y << 32) | r.x);
+          fx.add(((uint64_t)r.w << 32) | r.z);
+        }
+      }
+      if (MM) {
+        const uint32_t s0 = (uint32_t)((int32_t)r.y >> 31), s1 = (uint32_t)((int32_t)r.w >> 31);
+        const uint32_t h0 = r.y ^ (s0 | 0x80000000u), h1 = r.w ^ (s1 | 0x80000000u);
+        if (min(h0, h1) <= (uint32_t)((uint64_t)mn >> 32) || max(h0, h1) >= (uint32_t)((uint64_t)mx >> 32)) {
+          const U m0 = (U)(((uint64_t)h0 << 32) | (r.x ^ s0)), m1 = (U)(((uint64_t)h1 << 32) | (r.z ^ s1));
+          mn = min(mn, min(m0, m1));
+          mx = max(mx, max(m0, m1));
+        }
+      }
     }
   }
   // rows: the number of values this thread folded.
@@ -411,7 +445,7 @@ __device__ void merge_partials(const Partial* parts, int np, agg_scalar* out, ui
     // the oracle's own rounding of the exact sum (each at most 2^-53 of the
     // value); and a margin for the roundings of the bound's own sums.
     if (ops & (AGG_SUM | AGG_AVG)) {
-      const double units = acc.E ? ldexp((sizeof(typename Traits<DT>::T) == 8 ? 3.0 : 5.0) * (double)count,
+      const double units = acc.E > kFixFirst ? ldexp((sizeof(typename Traits<DT>::T) == 8 ? 3.0 : 5.0) * (double)count,
                                          acc.E - 1075 - kFixGuard)
                                  : 0.0;
       r.err_bound = ((double)acc.eb + units + fabs(s) * (0x1p-52 + 0x1p-99) + 0x1p-1072) * (1.0 + 0x1p-40);

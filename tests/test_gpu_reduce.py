@@ -244,3 +244,24 @@ def test_error_bound_of_integer_and_nonfinite_columns():
     z = np.arange(1000, dtype=np.float64)
     r = _scalar(z, agg.AGG_MIN | agg.AGG_MAX)
     assert r.err_bound == 0.0  # no SUM asked
+
+
+@pytest.mark.parametrize("below", [30, 31, 32, 33])
+@pytest.mark.parametrize("top", [2.0 ** -1000, 1.0, 2.0 ** 1000])
+def test_float64_rows_at_the_edge_of_the_fixed_point_window(below, top):
+    """Rows 30 to 33 binades below the largest, a pair of neighbours on either side of
+    the window, with zeros, subnormals and both signs among them."""
+    rng = np.random.default_rng(below)
+    n = 200_003
+    x = top * (1.0 + rng.random(n)) * rng.choice([-1.0, 1.0], n)
+    x[rng.random(n) < 0.5] *= 2.0 ** -below
+    x[::11] = 0.0
+    x[::13] = -0.0
+    x[5::17] = 5e-324
+    x[7::19] = -2.0 ** -1022
+    r = _scalar(x)
+    ref = math.fsum(x)
+    # three units a row at most; the unit is 2^-84 or 2^-83 of the power of two above the largest row
+    assert abs(r.sum_f - ref) <= 6.0 * n * 2.0 ** -83 * float(np.abs(x).max()) + 2.0 ** -52 * abs(ref)
+    assert abs(r.sum_f - ref) <= r.err_bound
+    assert r.min_f == x.min() and r.max_f == x.max()
