@@ -573,7 +573,8 @@ class HashRun {
       note_launch();
     } else if (ranked) {
       KernelPtr rk = pick_rank(vdt_, mm_);
-      const size_t sm = ((size_t)d + 4) * 4;
+      // in steps of 4 KB, so that the cached occupancy has 33 entries and not one for every group count
+      const size_t sm = (((size_t)d + 4) * 4 + 4095) & ~size_t(4095);
       (void)occupancy(rk, kRankThreads, sm);  // sets the kernel's shared-memory limit
       void* args[] = {&mem_, &k0, &s0, &o};
       e = cudaLaunchKernel(rk, dim3(rgrid), dim3(kRankThreads), args, sm, s_);
