@@ -23,9 +23,10 @@
 // is deterministic for a given grid. Measured against float64 TwoSum merges in
 // every shuffle step: 2^20 int32 rows 17.7 -> 8.7 us a call, 10^8 float64
 // rows 207 -> 178 us (with the scale started from the warp's first rows), 167 us
-// with two rows sharing the fast-path and MIN/MAX tests (SUM alone 131 -> 125;
-// bound by integer issue: five blocks a SM with 48 registers, no spill, take the
-// same 167 us).
+// with two rows sharing the fast-path and MIN/MAX tests (SUM alone 131 -> 125),
+// 155 us with the extremes shared by the warp after each iteration (a thread of
+// 430 rows moves its own a dozen times, and each time its warp goes along).
+// Bound by integer issue; five blocks a SM (48 registers, no spill) take 157 us.
 //
 // Error bound of a float SUM. It adds up the roundings that can occur: per
 // thread, those of the compensation word of a float32 pair (each at most 2^-24
@@ -80,6 +81,9 @@ __global__ void __launch_bounds__(kBlock, DT == AGG_I64 && MM ? 4 : 6) reduce_sc
       for (int u = 0; u < kUnroll; ++u)
         if (u * kBlock < left) a.fold_vec(r[u]);
       rows += EPV * (uint32_t)((left + kBlock - 1) / kBlock);
+      if constexpr (DT == AGG_F64 && MM) {  // when every lane has a next iteration
+        if (base + stride + (31 - (int)(threadIdx.x & 31)) < nv) a.share_extremes();
+      }
     }
   }
   Partial p;

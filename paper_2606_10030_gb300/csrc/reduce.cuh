@@ -314,6 +314,16 @@ struct Acc<DT, SUM, MM, true> {
       }
     }
   }
+  // float64 MIN/MAX, all lanes of the warp: every lane's extremes take the
+  // warp's high words, with low words that no value of theirs lies beyond (the
+  // lane that holds the warp's extreme keeps it). Only rows that may move the
+  // warp's extremes then pass the filter, not all that move one lane's.
+  __device__ __forceinline__ void share_extremes() {
+    const uint32_t lo = __reduce_min_sync(0xffffffffu, (uint32_t)((uint64_t)mn >> 32));
+    const uint32_t hi = __reduce_max_sync(0xffffffffu, (uint32_t)((uint64_t)mx >> 32));
+    mn = min(mn, (U)(((uint64_t)lo << 32) | 0xFFFFFFFFull));
+    mx = max(mx, (U)((uint64_t)hi << 32));
+  }
   // rows: the number of values this thread folded.
   __device__ void to_partial(Partial& p, uint32_t rows) const {
     p = Partial{};

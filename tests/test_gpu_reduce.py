@@ -265,3 +265,27 @@ def test_float64_rows_at_the_edge_of_the_fixed_point_window(below, top):
     assert abs(r.sum_f - ref) <= 6.0 * n * 2.0 ** -83 * float(np.abs(x).max()) + 2.0 ** -52 * abs(ref)
     assert abs(r.sum_f - ref) <= r.err_bound
     assert r.min_f == x.min() and r.max_f == x.max()
+
+
+@pytest.mark.parametrize("n", [1_867_775, 1_867_776, 1_867_779, 5_000_003])
+@pytest.mark.parametrize("kind", ["ascending", "descending", "constant", "one_high_word", "infinite", "zeros"])
+def test_float64_extremes_shared_by_a_warp(n, kind):
+    """Columns of one to several scan iterations a thread (and one row more or less),
+    whose extremes move with every row, tie, or share their high word."""
+    rng = np.random.default_rng(n)
+    x = np.arange(n, dtype=np.float64) - n / 2
+    if kind == "descending":
+        x = x[::-1].copy()
+    elif kind == "constant":
+        x[:] = -3.25
+    elif kind == "one_high_word":
+        x = np.float64(-1.5) + rng.integers(0, 1 << 20, n) * 2.0 ** -52
+    elif kind == "infinite":
+        x[rng.integers(0, n, 3)] = -np.inf
+        x[-1] = np.inf
+    elif kind == "zeros":
+        x = np.where(rng.random(n) < 0.5, 0.0, -0.0)
+    col = torch.from_numpy(x).cuda()
+    for ops in (agg.AGG_ALL, agg.AGG_MIN | agg.AGG_MAX):
+        r = agg.decode_scalar(agg.agg_reduce(col, ops))
+        assert r.min_f == x.min() and r.max_f == x.max()
