@@ -836,16 +836,26 @@ __device__ __forceinline__ void add96(uint32_t& a0, uint32_t& a1, uint32_t& a2, 
 }
 
 // The fixed-point sum top:w1:w0 (float64) or top:w0 (float32) of a window as a
-// float64: two roundings, then an exact scaling.
+// float64. float32: one rounding (both words are float64 integers). float64: the
+// magnitude's low word is rounded, then the whole, each to 2^-53 of the sum (of
+// the two's complement itself, a small negative sum's low word lies just below
+// 2^64 and would be rounded to multiples of 2^11 units); a single value has no
+// bits below its word's 53 and is exact. Then an exact scaling.
 template <int DT>
 __device__ __forceinline__ double fixed_to_double(int ebase, int64_t top, uint32_t w1, uint32_t w0) {
   if (DT == AGG_F32) {
     const double s = __hiloint2double((ebase - 150 + 1023) << 20, 0);
     return fma((double)top, 4294967296.0, (double)w0) * s;
   }
-  const double d = fma((double)top, 18446744073709551616.0, (double)(((unsigned long long)w1 << 32) | w0));
+  const uint64_t neg = (uint64_t)(top >> 63);  // all ones for a negative sum
+  uint64_t lo = (((uint64_t)w1 << 32) | w0) ^ neg;
+  uint64_t hi = (uint64_t)top ^ neg;
+  lo -= neg;
+  hi += neg != 0 && lo == 0 ? 1u : 0u;
+  const double d = fma((double)hi, 18446744073709551616.0, (double)lo);
   const int k = (ebase - 1075) / 2;  // in two steps, so that neither factor leaves the normal range
-  return d * __hiloint2double((k + 1023) << 20, 0) * __hiloint2double((ebase - 1075 - k + 1023) << 20, 0);
+  const double m = d * __hiloint2double((k + 1023) << 20, 0) * __hiloint2double((ebase - 1075 - k + 1023) << 20, 0);
+  return neg != 0 ? -m : m;
 }
 
 // What a row's value exceeds its sum term by (mod 2^64).
