@@ -17,23 +17,24 @@
 //   float64   a 128-bit fixed-point integer at the scale of the largest
 //             exponent seen (integer operations only: GB300 issues few
 //             float64 operations), uint64 images for min/max.
-// Float sums leave the threads as 128-bit fixed-point numbers (Fix128), and
-// warps, blocks and the grid merge them with integer additions; one thread
-// converts the total to float64 at the end. The order is fixed, so the result
-// is deterministic for a given grid. Measured against float64 TwoSum merges in
-// every shuffle step: 2^20 int32 rows 17.7 -> 8.7 us a call, 10^8 float64
-// rows 207 -> 178 us (with the scale started from the warp's first rows), 167 us
-// with two rows sharing the fast-path and MIN/MAX tests (SUM alone 131 -> 125),
-// 155 us with the extremes shared by the warp after each iteration (a thread of
-// 430 rows moves its own a dozen times, and each time its warp goes along).
-// Bound by integer issue; five blocks a SM (48 registers, no spill) take 157 us.
+// Float sums leave the threads as 128-bit fixed-point numbers (Fix128) with what
+// lies below their unit beside them in float64, and warps, blocks and the grid
+// merge them with integer additions; one thread converts the total to float64 at
+// the end. The order is fixed, so the result is deterministic for a given grid.
+// Measured against float64 TwoSum merges in every shuffle step: 2^20 int32 rows
+// 17.7 -> 8.7 us a call, 10^8 float64 rows 207 -> 158 us (with the scale started
+// from the warp's first rows, two rows sharing the fast-path and MIN/MAX tests,
+// SUM alone 168 -> 127, and the extremes shared by the warp after each iteration:
+// a thread of 430 rows moves its own a dozen times, and each time its warp goes
+// along). Rows outside the window cost more: exponents uniform over 60 binades
+// 408 -> 367 us, 98% zeros 366 -> 207 us. Bound by integer issue.
 //
 // Error bound of a float SUM. It adds up the roundings that can occur: per
 // thread, those of the compensation word of a float32 pair (each at most 2^-24
-// of the word's new value, tracked as the word's largest magnitude); the
-// fixed-point units lost (less than one per add, rescale or merge); the final
-// rounding of hi + lo and the oracle's own rounding of the exact sum, so that
-// |sum_f - (exact sum rounded to float64)| <= err_bound.
+// of the word's new value, tracked as the word's largest magnitude); what is
+// rounded or lost below the fixed-point unit (at most 2^-30 of it a row); the
+// final rounding of the sum and the oracle's own rounding of the exact sum, so
+// that |sum_f - (exact sum rounded to float64)| <= err_bound.
 #include <map>
 #include <mutex>
 
@@ -43,10 +44,11 @@ namespace agg {
 
 // The scan. Rows [0, head) and the ragged tail are folded with scalar loads by
 // the first threads of the grid; the 16-byte-aligned body with vector loads.
-// Six blocks a SM (40 registers) keep 98 KB of loads in flight a SM; int64
-// MIN/MAX needs 54 registers and runs four.
+// Six blocks a SM (40 registers, at most 18 bytes spilled) keep 98 KB of loads in
+// flight a SM; int64 MIN/MAX needs 54 registers and runs four, float64 sums run
+// five (48 registers, no spill; six spill 126 bytes: 160 us, not 158).
 template <int DT, bool SUM, bool MM>
-__global__ void __launch_bounds__(kBlock, DT == AGG_I64 && MM ? 4 : 6) reduce_scan(const typename Traits<DT>::T* __restrict__ col,
+__global__ void __launch_bounds__(kBlock, DT == AGG_I64 && MM ? 4 : DT == AGG_F64 && SUM ? 5 : 6) reduce_scan(const typename Traits<DT>::T* __restrict__ col,
                                                       int64_t n, int64_t head, Partial* __restrict__ parts,
                                                       int part_base, unsigned* ticket, agg_scalar* out,
                                                       uint32_t ops, int64_t count_total, int finalize) {
@@ -69,7 +71,8 @@ __global__ void __launch_bounds__(kBlock, DT == AGG_I64 && MM ? 4 : 6) reduce_sc
       // warp through the slow path some hundred times
       const int64_t i0 = (int64_t)blockIdx.x * kBlock * kUnroll + threadIdx.x;
       const uint4 r = i0 < nv ? ld_stream_v4(v + i0) : make_uint4(0, 0, 0, 0);
-      a.fx.start(__reduce_max_sync(0xffffffffu, max((r.y >> 20) & 0x7FFu, (r.w >> 20) & 0x7FFu)));
+      const uint32_t own = max((r.y >> 20) & 0x7FFu, (r.w >> 20) & 0x7FFu);
+      a.fx.start(__reduce_max_sync(0xffffffffu, own), own);
     }
     for (int64_t base = (int64_t)blockIdx.x * kBlock * kUnroll + threadIdx.x; base < nv; base += stride) {
       const int left = (int)min(nv - base, (int64_t)kUnroll * kBlock);  // vector u exists when u * kBlock < left

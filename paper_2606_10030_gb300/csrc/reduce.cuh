@@ -17,14 +17,17 @@ namespace agg {
 // of Fix128 at the scale of exponent E, so that warps, blocks and the grid
 // merge with integer additions: GB300 issues few float64 operations, and a
 // float64 TwoSum in every shuffle step made a 2^20-row int32 scan 17 us long
-// and put 40 us on every float64 scan.
+// and put 40 us on every float64 scan. What a merge shifts below the unit goes
+// to rest, in float64: nothing in a column whose rows lie within some 30
+// binades of each other, and in any other what keeps a sum right whose largest
+// rows cancel.
 struct Partial {
   uint64_t w0, w1;
   uint64_t mn, mx;   // order-preserving images of min / max
-  int32_t E;         // exponent field the fixed-point sum is scaled to (0: no value yet)
-  uint32_t special;  // float: kPosInf | kNegInf | kNan seen
+  double rest;       // float: the sum's part below the unit of w1:w0
+  int16_t E;         // exponent field the fixed-point sum is scaled to (0: no value yet)
+  uint16_t special;  // float: kPosInf | kNegInf | kNan seen
   float eb;          // float32: bound on the roundings of the threads' compensation words
-  uint32_t pad;
 };
 static_assert(sizeof(Partial) == 48, "partials of the static scratch");
 constexpr uint32_t kPosInf = 1, kNegInf = 2, kNan = 4;
@@ -90,9 +93,9 @@ template <> struct FpImg<double> {
 // (hi:lo) x 2^(E - 1075 - kFixGuard). A row with significand m (53 bits,
 // implicit bit included) and exponent field e >= 1 is worth m x 2^(e - 1075),
 // i.e. m shifted left by kFixGuard - (E - e) units. Rows more than kFixGuard
-// binades below E keep their bits above the unit (each loses less than
-// 2^(E - 1075 - kFixGuard), 2^-83 of the largest row); a row with a larger
-// exponent shifts the sum right (again less than a unit lost). Sums of up to
+// binades below E reach into a further word ext, whose unit is 2^-64 of that of
+// lo (a row loses less than that, 2^-147 of the largest row); a row with a larger
+// exponent shifts the sum right (again less than a unit of ext lost). Sums of up to
 // 2^43 rows per thread cannot overflow (|m x 2^kFixGuard| < 2^84). A guard of
 // 31 bits keeps the fast path's shift below one word. Infinities and NaNs are noted
 // on the side, so that a column holding one sums to a non-finite value.
@@ -104,8 +107,15 @@ template <> struct FpImg<double> {
 constexpr int kFixGuard = 31;
 constexpr int kFixFirst = kFixGuard + 1;
 
+// x 2^k for -1140 <= k <= 1022, rounded at most once (two normal factors).
+__device__ __forceinline__ double scaled(double x, int k) {
+  const int h = k / 2;
+  return x * __hiloint2double((h + 1023) << 20, 0) * __hiloint2double((k - h + 1023) << 20, 0);
+}
+
 struct Fix128 {
   uint64_t lo, hi;
+  uint64_t ext;   // the bits below lo's unit (slow path only)
   uint32_t nneg;  // negative rows added on the fast path as ~v, each still owing +1
   int E;
   uint32_t base;  // (E - kFixGuard) << 20: a row's high word minus this holds the row's shift
@@ -113,14 +123,20 @@ struct Fix128 {
   __device__ void init() {
     lo = 0;
     hi = 0;
+    ext = 0;
     nneg = 0;
     E = kFixFirst;
     base = 1u << 20;
     special = 0;
   }
-  // Scale for rows of exponent fields up to ef + 1 (the sum so far is zero or exact).
-  __device__ __forceinline__ void start(uint32_t ef) {
-    if (ef > 0 && ef < 0x7FEu && (int)ef >= E) rescale((int)ef + 1);
+  // Scale for rows of exponent fields up to ef + 1, where the thread's own first
+  // rows reach up to own: at most 64 binades above those, so that ext still holds
+  // every bit that a scale of the thread's own rows would (the sum so far is zero
+  // or exact).
+  __device__ __forceinline__ void start(uint32_t ef, uint32_t own) {
+    if (ef == 0x7FFu) return;
+    ef = min(min(ef, own + 63u), 0x7FDu);
+    if (ef > 0 && (int)ef >= E) rescale((int)ef + 1);
   }
   // -v = ~v + 1: the fast path adds ~v and counts the +1s, added here.
   __device__ __forceinline__ void fold_neg() {
@@ -128,12 +144,9 @@ struct Fix128 {
     hi += lo < nneg ? 1ull : 0ull;
     nneg = 0;
   }
-  // (vhi:vlo) >> k for k >= 1, rounding toward minus infinity (less than one unit).
+  // (vhi:vlo) >> k for 1 <= k < 127, rounding toward minus infinity (less than one unit).
   __device__ static __forceinline__ void shift_right(uint64_t& vlo, uint64_t& vhi, int k) {
-    if (k >= 127) {
-      vlo = (int64_t)vhi < 0 ? ~0ull : 0ull;
-      vhi = vlo;
-    } else if (k >= 64) {
+    if (k >= 64) {
       vlo = (uint64_t)((int64_t)vhi >> (k - 64));
       vhi = (uint64_t)((int64_t)vhi >> 63);
     } else {
@@ -143,7 +156,20 @@ struct Fix128 {
   }
   __device__ __forceinline__ void rescale(int e) {  // e > E
     fold_neg();
-    shift_right(lo, hi, e - E);
+    int k = e - E;
+    if (k >= 191) {  // nothing of the sum reaches ext's unit
+      ext = lo = hi = 0;
+      k = 0;
+    }
+    for (; k >= 64; k -= 64) {
+      ext = lo;
+      lo = hi;
+      hi = (uint64_t)((int64_t)hi >> 63);
+    }
+    if (k > 0) {
+      ext = (ext >> k) | (lo << (64 - k));
+      shift_right(lo, hi, k);
+    }
     E = e;
     base = (uint32_t)(e - kFixGuard) << 20;
   }
@@ -180,45 +206,59 @@ struct Fix128 {
         : "r"(x0), "r"(x1), "r"(x2), "r"(x3));
     nneg -= s;
   }
+  // Any row. (Not through add_fast where that would do: a warp with a row outside
+  // the window would take both paths one after the other.)
   __device__ __forceinline__ void add(uint64_t u) {
-    const uint32_t uh = (uint32_t)(u >> 32), ul = (uint32_t)u;
-    const uint32_t x = rel(uh);
-    if ((x & kFixOut) == 0u) {
-      add_fast(uh, ul, x);
-      return;
-    }
+    const uint32_t uh = (uint32_t)(u >> 32);
+    uint32_t ml = (uint32_t)u;
+    if (((uh << 1) | ml) == 0u) return;
     const int ef = (int)((uh >> 20) & 0x7FFu);
-    fold_neg();
-    if (ef == 0x7FF) {  // infinity or NaN
-      special |= (u & 0x000FFFFFFFFFFFFFull) ? kNan : (int64_t)u < 0 ? kNegInf : kPosInf;
-      return;
+    if (ef > E) {
+      if (ef == 0x7FF) {  // infinity or NaN
+        special |= (u & 0x000FFFFFFFFFFFFFull) ? kNan : (int64_t)u < 0 ? kNegInf : kPosInf;
+        return;
+      }
+      rescale(ef);
     }
-    const int e = ef > 0 ? ef : 1;  // subnormals: exponent 1, no implicit bit
-    const uint64_t m = (u & 0x000FFFFFFFFFFFFFull) | ((uint64_t)(ef > 0) << 52);
-    if (e > E) rescale(e);
-    const int d = E - e;
-    uint64_t vlo, vhi;
-    if (d <= kFixGuard) {
-      const int sh = kFixGuard - d;  // 0 .. kFixGuard
-      vlo = m << sh;
-      vhi = sh > 0 ? m >> (64 - sh) : 0ull;
-    } else {
-      const int r = d - kFixGuard;
-      vlo = r < 64 ? m >> r : 0ull;
-      vhi = 0ull;
+    // The significand m (subnormals: exponent 1, no implicit bit) in units of ext
+    // is m shifted left by kFixGuard + 64 - (E - e): three words x0, x1, x2 at
+    // word q of the six words hi:lo:ext.
+    uint32_t mh = (uh & 0x000FFFFFu) | (ef > 0 ? 0x00100000u : 0u);
+    int sh = kFixGuard + 64 - E + max(ef, 1);
+    if (sh < 0) {
+      const uint64_t m = sh > -64 ? (((uint64_t)mh << 32) | ml) >> -sh : 0ull;
+      ml = (uint32_t)m;
+      mh = (uint32_t)(m >> 32);
+      sh = 0;
     }
-    if ((int64_t)u < 0) {  // two's-complement negation of vhi:vlo
-      vlo = ~vlo + 1ull;
-      vhi = ~vhi + (vlo == 0ull ? 1ull : 0ull);
-    }
-    lo += vlo;
-    hi += vhi + (lo < vlo ? 1ull : 0ull);
+    const int q = sh >> 5;  // 0 to 2
+    const uint32_t s = (uint32_t)((int32_t)uh >> 31);  // a negative row: the complement, plus one
+    const uint32_t x0 = __funnelshift_l(0u, ml, sh) ^ s;
+    const uint32_t x1 = __funnelshift_l(ml, mh, sh) ^ s;
+    const uint32_t x2 = __funnelshift_l(mh, 0u, sh) ^ s;
+    asm("{\n\t.reg .u32 t, a0, a1, a2, a3, a4, a5;\n\t"
+        "mov.b64 {a0, a1}, %0;\n\t"
+        "mov.b64 {a2, a3}, %1;\n\t"
+        "mov.b64 {a4, a5}, %2;\n\t"
+        "add.cc.u32 t, %8, %8;\n\t"  // carry: the sign
+        "addc.cc.u32 a0, a0, %3;\n\t"
+        "addc.cc.u32 a1, a1, %4;\n\t"
+        "addc.cc.u32 a2, a2, %5;\n\t"
+        "addc.cc.u32 a3, a3, %6;\n\t"
+        "addc.cc.u32 a4, a4, %7;\n\t"
+        "addc.u32 a5, a5, %8;\n\t"
+        "mov.b64 %0, {a0, a1};\n\t"
+        "mov.b64 %1, {a2, a3};\n\t"
+        "mov.b64 %2, {a4, a5};\n\t}"
+        : "+l"(ext), "+l"(lo), "+l"(hi)
+        : "r"(q == 0 ? x0 : s), "r"(q == 0 ? x1 : q == 1 ? x0 : s), "r"(q == 0 ? x2 : q == 1 ? x1 : x0),
+          "r"(q == 1 ? x2 : q == 2 ? x1 : s), "r"(q == 2 ? x2 : s), "r"(s));
   }
 };
 
-// The sum of a partial as an unevaluated float64 pair (rel. error about 2^-106
-// before scaling): the 128-bit integer in three chunks that float64 holds
-// exactly, added with TwoSum, then scaled by 2^(E - 1075 - kFixGuard).
+// The sum of a partial without its rest, as an unevaluated float64 pair (rel.
+// error about 2^-106 before scaling): the 128-bit integer in three chunks that
+// float64 holds exactly, added with TwoSum, then scaled by 2^(E - 1075 - kFixGuard).
 __device__ inline void fix_to_pair(const Partial& p, double& h, double& l) {
   const uint64_t lo = p.w0, hi = p.w1;
   const uint64_t m43 = (1ull << 43) - 1ull;
@@ -342,8 +382,14 @@ struct Acc<DT, SUM, MM, true> {
       f.fold_neg();
       p.w0 = f.lo;
       p.w1 = f.hi;
-      p.E = f.E;
-      p.special = f.special;
+      if (f.ext != 0) {  // the part below the unit has the sum's sign, so that it is no larger than the sum
+        const bool neg = (int64_t)f.hi < 0;
+        if (neg && ++p.w0 == 0) ++p.w1;  // toward zero
+        p.rest = scaled((double)(neg ? 0ull - f.ext : f.ext), f.E - 1075 - kFixGuard - 64);
+        if (neg) p.rest = -p.rest;
+      }
+      p.E = (int16_t)f.E;
+      p.special = (uint16_t)f.special;
     }
     p.mn = mn == (U)~(U)0 ? ~0ull : (uint64_t)mn;
     p.mx = mx;
@@ -353,20 +399,52 @@ struct Acc<DT, SUM, MM, true> {
 // ---------------------------------------------------------------------------
 // Warp / block reduction of Partial values (fixed shuffle tree).
 // ---------------------------------------------------------------------------
+// w1:w0 at the scale of E moved to that of E + k (1 <= k), toward zero: what falls
+// below the new unit is returned, rounded to float64. (It has the sum's sign: a
+// sum below the unit is returned whole, not as a unit and what that exceeds it by.)
+__device__ __forceinline__ double lower_scale(uint64_t& w0, uint64_t& w1, int E, int k) {
+  const bool neg = (int64_t)w1 < 0;
+  uint64_t l0 = neg ? 0ull - w0 : w0, l1 = neg ? ~w1 + (w0 == 0 ? 1ull : 0ull) : w1;
+  w0 = l0;
+  w1 = l1;
+  if (k < 64) {
+    l0 &= (1ull << k) - 1ull;
+    l1 = 0;
+    w0 = (w0 >> k) | (w1 << (64 - k));
+    w1 >>= k;
+  } else if (k < 128) {
+    l1 &= (1ull << (k - 64)) - 1ull;
+    w0 = w1 >> (k - 64);
+    w1 = 0;
+  } else {
+    w0 = w1 = 0;
+  }
+  if (neg) {
+    w0 = 0ull - w0;
+    w1 = ~w1 + (w0 == 0 ? 1ull : 0ull);
+  }
+  if ((l0 | l1) == 0) return 0.0;
+  const double d = scaled(fma((double)l1, 18446744073709551616.0, (double)l0), E - 1075 - kFixGuard);
+  return neg ? -d : d;
+}
+
+// The sum of a partial moved to the scale of exponent E >= its own.
+__device__ __forceinline__ void raise_scale(Partial& p, int E) {
+  if (p.E == E) return;
+  const double d = lower_scale(p.w0, p.w1, p.E, E - p.E);
+  if (d != 0.0) p.rest += d;
+  p.E = (int16_t)E;
+}
+
 template <bool FP>
-__device__ __forceinline__ void combine(Partial& a, const Partial& b) {
+__device__ __forceinline__ void combine(Partial& a, Partial b) {
   if (FP) {
-    // the sum of the smaller exponent is shifted to the other's scale (less
-    // than one unit lost), then added
-    uint64_t blo = b.w0, bhi = b.w1;
-    if (b.E > a.E) {
-      Fix128::shift_right(a.w0, a.w1, b.E - a.E);
-      a.E = b.E;
-    } else if (b.E < a.E) {
-      Fix128::shift_right(blo, bhi, a.E - b.E);
-    }
-    a.w0 += blo;
-    a.w1 += bhi + (a.w0 < blo ? 1ull : 0ull);
+    const int E = max(a.E, b.E);
+    raise_scale(a, E);
+    raise_scale(b, E);
+    a.w0 += b.w0;
+    a.w1 += b.w1 + (a.w0 < b.w0 ? 1ull : 0ull);
+    if (b.rest != 0.0) a.rest += b.rest;
     a.special |= b.special;
     a.eb = __fadd_ru(a.eb, b.eb);
   } else {
@@ -382,34 +460,50 @@ __device__ __forceinline__ Partial empty_partial() {
   return p;
 }
 
-template <bool FP>
-__device__ __forceinline__ Partial shfl_xor(const Partial& p, int m) {
-  Partial q{};
-  q.w0 = __shfl_xor_sync(0xffffffffu, p.w0, m);
+__device__ __forceinline__ uint64_t warp_min64(uint64_t v) {  // the high words' minimum, then the low words of the lanes holding it
+  const uint32_t h = __reduce_min_sync(0xffffffffu, (uint32_t)(v >> 32));
+  return ((uint64_t)h << 32) | __reduce_min_sync(0xffffffffu, (uint32_t)(v >> 32) == h ? (uint32_t)v : 0xFFFFFFFFu);
+}
+
+// The lanes' partials (the first LANES of them hold one), in lane 0. Floats: all
+// lanes take the largest exponent's scale first, so that the sums are plain
+// integer additions (with a shift in every step, the end of a float scan was 7 us
+// longer); the float64 parts below the unit are added only when a lane has one.
+template <bool FP, int LANES>
+__device__ __forceinline__ void warp_combine(Partial& p) {
+  constexpr unsigned kAll = 0xffffffffu;
   if (FP) {
-    q.w1 = __shfl_xor_sync(0xffffffffu, p.w1, m);
-    q.E = __shfl_xor_sync(0xffffffffu, p.E, m);
-    q.special = __shfl_xor_sync(0xffffffffu, p.special, m);
-    q.eb = __shfl_xor_sync(0xffffffffu, p.eb, m);
+    raise_scale(p, (int)__reduce_max_sync(kAll, (uint32_t)p.E));
+    p.special = (uint16_t)__reduce_or_sync(kAll, p.special);
+    if (__any_sync(kAll, p.rest != 0.0)) {
+#pragma unroll 1
+      for (int m = LANES / 2; m >= 1; m >>= 1) p.rest += __shfl_xor_sync(kAll, p.rest, m);
+    }
   }
-  q.mn = __shfl_xor_sync(0xffffffffu, p.mn, m);
-  q.mx = __shfl_xor_sync(0xffffffffu, p.mx, m);
-  return q;
+#pragma unroll
+  for (int m = LANES / 2; m >= 1; m >>= 1) {
+    const uint64_t b0 = __shfl_xor_sync(kAll, p.w0, m);
+    p.w0 += b0;
+    if (FP) {
+      p.w1 += __shfl_xor_sync(kAll, p.w1, m) + (p.w0 < b0 ? 1ull : 0ull);
+      p.eb = __fadd_ru(p.eb, __shfl_xor_sync(kAll, p.eb, m));
+    }
+  }
+  p.mn = warp_min64(p.mn);
+  p.mx = ~warp_min64(~p.mx);
 }
 
 // Block-wide reduction; the result is valid in thread 0.
 template <bool FP, int BLOCK>
 __device__ Partial block_reduce(Partial p) {
   __shared__ Partial sm[BLOCK / 32];
-#pragma unroll
-  for (int m = 16; m >= 1; m >>= 1) combine<FP>(p, shfl_xor<FP>(p, m));
+  warp_combine<FP, 32>(p);
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
   if (l == 0) sm[w] = p;
   __syncthreads();
   if (w == 0) {
     p = l < BLOCK / 32 ? sm[l] : empty_partial();
-#pragma unroll
-    for (int m = BLOCK / 64; m >= 1; m >>= 1) combine<FP>(p, shfl_xor<FP>(p, m));
+    warp_combine<FP, BLOCK / 32>(p);
   }
   return p;
 }
@@ -445,20 +539,26 @@ __device__ void merge_partials(const Partial* parts, int np, agg_scalar* out, ui
     double hi, lo;
     fix_to_pair(acc, hi, lo);
     double s = hi + lo;
+    const double parts = fabs(hi) + fabs(acc.rest);
+    if (acc.rest != 0.0 && isfinite(s)) {
+      double e;
+      two_sum(hi, acc.rest, s, e);
+      s += e + lo;
+    }
     r.sum_i = 0;
     r.sum_f = s;
     // Bound on |s - exact sum|: the threads' compensation words (float32); the
-    // fixed-point units lost, less than one per add, per rescale and per merge
-    // of a thread's sum (float64: at most three a row; float32: a thread that
-    // folded a row adds two words, so at most five a row); fix_to_pair (under
-    // 2^-104 of the sum, and the subnormal range); the rounding of hi + lo and
-    // the oracle's own rounding of the exact sum (each at most 2^-53 of the
-    // value); and a margin for the roundings of the bound's own sums.
+    // rounding of what is below the unit, a thread's ext word and the part that
+    // a merge shifts out (each less than a unit, 2^-52 of it lost), and of the
+    // additions to rest (2^-53 of at most a unit per row merged, at a depth of
+    // less than 2^20): 2^-30 of a unit a row holds all of it, and the rows'
+    // 2^-64; fix_to_pair and the addition of rest (under 2^-100 of the parts,
+    // and the subnormal range); the rounding of the result and the oracle's own
+    // rounding of the exact sum (each at most 2^-53 of the value); and a margin
+    // for the roundings of the bound's own sums.
     if (ops & (AGG_SUM | AGG_AVG)) {
-      const double units = acc.E > kFixFirst ? ldexp((sizeof(typename Traits<DT>::T) == 8 ? 3.0 : 5.0) * (double)count,
-                                         acc.E - 1075 - kFixGuard)
-                                 : 0.0;
-      r.err_bound = ((double)acc.eb + units + fabs(s) * (0x1p-52 + 0x1p-99) + 0x1p-1072) * (1.0 + 0x1p-40);
+      const double units = acc.E > kFixFirst ? ldexp((double)count, acc.E - 1075 - kFixGuard - 30) : 0.0;
+      r.err_bound = ((double)acc.eb + units + fabs(s) * 0x1p-52 + parts * 0x1p-99 + 0x1p-1072) * (1.0 + 0x1p-40);
       // a column holding an infinity or a NaN has no finite bound
       if (acc.special || !isfinite(s) || !isfinite(r.err_bound)) r.err_bound = inf;
     }

@@ -63,3 +63,47 @@ def test_small_negative_groups_keep_their_bits(how, dt, rows_a_group):
         assert np.array_equal(res["avg"][small], want)
     else:
         assert np.all(np.abs(got - want) <= 3 * 2.0 ** -53 * np.abs(want))
+
+
+def scan(x, host):
+    if host:
+        return agg.agg_reduce_host(torch.from_numpy(x).pin_memory(), agg.AGG_ALL)
+    return agg.decode_scalar(agg.agg_reduce(torch.from_numpy(x).cuda(), agg.AGG_ALL))
+
+
+@pytest.mark.parametrize("host", [False, True])
+@pytest.mark.parametrize("small", ["ones", "normal"])
+@pytest.mark.parametrize("dt,big", [(np.float32, 1e30), (np.float64, 2.0 ** 100), (np.float64, 1e35), (np.float64, 1e300)])
+def test_scan_of_large_values_that_cancel(dt, big, small, host):
+    """Rows far apart cancel and leave the other rows' sum. A thread folds at most 24 of these rows (2^22
+    rows in at least 2^18 vectors' blocks). Of a thread that holds a large value, float64 rows lose what
+    lies below 2^-147 of it, float32 rows nothing (TwoSum); what the merges shift below the unit is
+    added in float64, at most 20 additions deep."""
+    n = 1 << 22
+    x = np.ones(n, dtype=dt)
+    if small == "normal":
+        x = np.random.default_rng(1).standard_normal(n).astype(dt)
+    x[12_345], x[n - 77] = big, -big
+    total = math.fsum(np.delete(x, [12_345, n - 77]).astype(np.float64))
+    a = float(np.abs(np.delete(x, [12_345, n - 77]).astype(np.float64)).sum())
+    lost = 0.0
+    if dt is np.float64:
+        lost = 48 * min(float(np.abs(x[np.abs(x) < big]).max()), big * 2.0 ** -146)
+    r = scan(x, host)
+    assert abs(r.sum_f - total) <= lost + (0.0 if small == "ones" else 20 * 2.0 ** -53 * a)
+    assert abs(r.sum_f - total) <= r.err_bound
+    assert np.isfinite(r.err_bound)
+
+
+@pytest.mark.parametrize("span", [10, 40, 90, 140, 400, 2000])
+def test_float64_scan_of_any_span_is_the_exact_sum(span):
+    """Exponents uniform over span binades: the sum differs from the exact one by its own rounding and
+    2^-100 of the largest rows, and the bound holds."""
+    rng = np.random.default_rng(span)
+    n = 1_000_003
+    x = rng.standard_normal(n) * np.exp2(rng.integers(-span // 2, span // 2 + 1, n).astype(float))
+    for y in (x, np.concatenate([x, -x[::-1][: n - 5]])):
+        ref = math.fsum(y)
+        r = scan(y, False)
+        assert abs(r.sum_f - ref) <= 2.0 ** -53 * abs(ref) + y.size * 2.0 ** -120 * float(np.abs(y).max())
+        assert abs(r.sum_f - ref) <= r.err_bound
