@@ -382,11 +382,9 @@ struct Acc<DT, SUM, MM, true> {
       f.fold_neg();
       p.w0 = f.lo;
       p.w1 = f.hi;
-      if (f.ext != 0) {  // the part below the unit has the sum's sign, so that it is no larger than the sum
-        const bool neg = (int64_t)f.hi < 0;
-        if (neg && ++p.w0 == 0) ++p.w1;  // toward zero
-        p.rest = scaled((double)(neg ? 0ull - f.ext : f.ext), f.E - 1075 - kFixGuard - 64);
-        if (neg) p.rest = -p.rest;
+      if (f.ext != 0) {  // to the nearest unit (see lower_scale)
+        if ((int64_t)f.ext < 0 && ++p.w0 == 0) ++p.w1;
+        p.rest = scaled((double)(int64_t)f.ext, f.E - 1075 - kFixGuard - 64);
       }
       p.E = (int16_t)f.E;
       p.special = (uint16_t)f.special;
@@ -399,31 +397,31 @@ struct Acc<DT, SUM, MM, true> {
 // ---------------------------------------------------------------------------
 // Warp / block reduction of Partial values (fixed shuffle tree).
 // ---------------------------------------------------------------------------
-// w1:w0 at the scale of E moved to that of E + k (1 <= k), toward zero: what falls
-// below the new unit is returned, rounded to float64. (It has the sum's sign: a
-// sum below the unit is returned whole, not as a unit and what that exceeds it by.)
+// w1:w0 at the scale of E moved to that of E + k (1 <= k), to the nearest unit: what
+// that leaves, half a unit at most, is returned, rounded to float64. (Rounded down,
+// what a small negative sum leaves would be nearly a unit, and its own bits lost.)
 __device__ __forceinline__ double lower_scale(uint64_t& w0, uint64_t& w1, int E, int k) {
-  const bool neg = (int64_t)w1 < 0;
-  uint64_t l0 = neg ? 0ull - w0 : w0, l1 = neg ? ~w1 + (w0 == 0 ? 1ull : 0ull) : w1;
-  w0 = l0;
-  w1 = l1;
-  if (k < 64) {
-    l0 &= (1ull << k) - 1ull;
-    l1 = 0;
-    w0 = (w0 >> k) | (w1 << (64 - k));
-    w1 >>= k;
-  } else if (k < 128) {
-    l1 &= (1ull << (k - 64)) - 1ull;
-    w0 = w1 >> (k - 64);
-    w1 = 0;
-  } else {
+  uint64_t l0, l1;  // what is left, two's complement
+  if (k < 127) {
+    const uint64_t h0 = k <= 64 ? 1ull << (k - 1) : 0ull, h1 = k > 64 ? 1ull << (k - 65) : 0ull;  // half a unit
+    w0 += h0;
+    w1 += h1 + (w0 < h0 ? 1ull : 0ull);
+    l0 = k < 64 ? w0 & ((1ull << k) - 1ull) : w0;
+    l1 = k > 64 ? w1 & ((1ull << (k - 64)) - 1ull) : 0ull;
+    Fix128::shift_right(w0, w1, k);
+    l1 -= h1 + (l0 < h0 ? 1ull : 0ull);
+    l0 -= h0;
+  } else {  // below half a unit
+    l0 = w0;
+    l1 = w1;
     w0 = w1 = 0;
   }
-  if (neg) {
-    w0 = 0ull - w0;
-    w1 = ~w1 + (w0 == 0 ? 1ull : 0ull);
-  }
   if ((l0 | l1) == 0) return 0.0;
+  const bool neg = (int64_t)l1 < 0;
+  if (neg) {
+    l0 = 0ull - l0;
+    l1 = ~l1 + (l0 == 0 ? 1ull : 0ull);
+  }
   const double d = scaled(fma((double)l1, 18446744073709551616.0, (double)l0), E - 1075 - kFixGuard);
   return neg ? -d : d;
 }
