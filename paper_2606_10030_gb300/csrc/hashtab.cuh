@@ -396,7 +396,7 @@ __device__ __forceinline__ void report_counts(const BuildArgs& a, const BlockCou
 // The window of a block or tile comes from 32 of its rows: int64: 2^32 values
 // from a base that holds the sampled range (aligned to 2^32 when the samples
 // share their high word, else centred); floats: up to 3 binades above the
-// largest sampled exponent.
+// largest exponent sampled (of 512 rows more when the 32 are zeros).
 // ---------------------------------------------------------------------------
 constexpr uint32_t kMiss = 0xFFFFFFFFu;  // no slot (yet)
 constexpr int64_t kEpochRows = 65532;    // rows a block folds between two moves of the cnt halves (a multiple of 4)
@@ -656,7 +656,7 @@ __device__ __forceinline__ Enc<DT> s_enc(const TAB& t, typename GV<DT>::T v) {
 
 // Sum of a float the window does not hold (zeros add nothing), into the fb words at a.
 template <int DT>
-__device__ __noinline__ void s_add_other(uint32_t a, typename GV<DT>::T v) {
+__device__ __forceinline__ void s_add_other(uint32_t a, typename GV<DT>::T v) {
   if (v == typename GV<DT>::T(0)) return;
   if constexpr (DT == AGG_F32) {
     float old, sum, err;
@@ -828,6 +828,8 @@ __device__ __forceinline__ void s_fold(const BuildArgs& a, const TAB& t, const u
 // frequent keys cause.
 // ---------------------------------------------------------------------------
 constexpr int kDominantRows = 16; // rows of one key (of 128) that make a reduced update pay
+constexpr int kDominantOther = 4; // of floats outside the window (compare-and-swap updates)
+                                  // (above 8 keys: 30 keys, float32 294 us with 4, 337 with 16)
 constexpr int kMaxWarpKeys = 8;   // keys reduced per warp and quad of rows, at most
 
 // a2:a1:a0 += v
@@ -875,7 +877,7 @@ __device__ __forceinline__ void warp_add32(uint32_t v, uint32_t& lo, uint32_t& c
 }
 
 // The warp reduces the rows marked in take (a 4-bit mask a lane; all of one
-// key, floats all in the window) and lane 0 adds them to the key's slot.
+// key, floats all zero or in the window) and lane 0 adds them to the key's slot.
 template <int DT, bool MM, class TAB>
 __device__ __forceinline__ void s_fold_warp_key(const BuildArgs& a, const TAB& t, uint32_t key,
                                                 const typename GV<DT>::T (&v)[4], uint32_t take) {
@@ -888,10 +890,12 @@ __device__ __forceinline__ void s_fold_warp_key(const BuildArgs& a, const TAB& t
   for (int r = 0; r < 4; ++r) {
     if (!((take >> r) & 1u)) continue;
     const Enc<DT> e = s_enc<DT>(t, v[r]);
-    asm("{add.cc.u32 %0, %0, %3; addc.cc.u32 %1, %1, %4; addc.u32 %2, %2, %5;}"
-        : "+r"(c0), "+r"(c1), "+r"(c2)
-        : "r"(e.e0), "r"(e.e1), "r"(e.e2));
-    if (is_float(DT)) add96(c0, c1, c2, e.neg >> 16);  // the +1 of a negative row's two's complement
+    if (!is_float(DT) || e.ok) {  // zeros add nothing
+      asm("{add.cc.u32 %0, %0, %3; addc.cc.u32 %1, %1, %4; addc.u32 %2, %2, %5;}"
+          : "+r"(c0), "+r"(c1), "+r"(c2)
+          : "r"(e.e0), "r"(e.e1), "r"(e.e2));
+      if (is_float(DT)) add96(c0, c1, c2, e.neg >> 16);  // the +1 of a negative row's two's complement
+    }
     if (MM) {
       if (is_wide(DT)) {
         const uint64_t m = GV<DT>::img(v[r]);
@@ -982,6 +986,61 @@ __device__ __forceinline__ void s_fold_warp_key(const BuildArgs& a, const TAB& t
   }
 }
 
+// The same for a key with floats outside the window: all of its rows as a
+// compensated float32 pair or a float64 sum, into the slot's fb words. (Row by row,
+// they are compare-and-swap loops on one address. 2^24 rows with exponents uniform
+// over 60 binades, SUM/COUNT: of 8 keys, float32 664 us, 306 so, float64 1621 and
+// 828; of 10^6 skewed keys, float32 1362 and 748, float64 5003 and 945.)
+template <int DT, bool MM>
+__device__ __noinline__ Partial4<DT> s_other_partial(typename GV<DT>::T v0, typename GV<DT>::T v1,
+                                                     typename GV<DT>::T v2, typename GV<DT>::T v3, uint32_t take) {
+  const typename GV<DT>::T v[4] = {v0, v1, v2, v3};
+  Partial4<DT> p = partial_of<DT, MM>(v, take);
+  warp_reduce_partial<DT, MM>(p);
+  return p;
+}
+
+template <int DT, bool MM, class TAB>
+__device__ __forceinline__ void s_fold_warp_other(const BuildArgs& a, const TAB& t, uint32_t key,
+                                                  const typename GV<DT>::T (&v)[4], uint32_t take) {
+  using L = typename TAB::L;
+  const Partial4<DT> p = s_other_partial<DT, MM>(v[0], v[1], v[2], v[3], take);
+  if ((threadIdx.x & 31) != 0) return;
+  const uint32_t j = key == 0xFFFFFFFFu ? t.side() : s_place(key + 1, t);
+  if (j == kMiss) {
+    GPart g[1];
+    g[0].key = key;
+    g[0].cnt = p.cnt;
+    g[0].sum = (unsigned long long)__double_as_longlong(is_f32(DT) ? (double)p.fs + (double)p.fc : p.ds);
+    if (MM) {
+      g[0].nmn = ~g_img_of<DT>(p.mn);
+      g[0].mx = g_img_of<DT>(p.mx);
+    }
+    g_merge<DT, MM, 1>(a, g, 1u);
+    return;
+  }
+  sm_add<L::kCnt>(j, p.cnt);
+  const uint32_t jf = j + (j - t.b0) + L::kFb;
+  if constexpr (is_f32(DT)) {
+    s_add_other<DT>(jf, p.fs);
+    if (p.fc != 0.f) asm volatile("red.shared.add.f32 [%0+4], %1;" ::"r"(jf), "f"(p.fc));
+    if constexpr (MM) {
+      const uint32_t jm = j + (j - t.b0);
+      const uint2 q = sm_ld2<L::kMM>(jm);
+      sm_raise<L::kMM>(jm, ~p.mn, q.x);
+      sm_raise<L::kMM + 4>(jm, p.mx, q.y);
+    }
+  } else {
+    s_add_other<DT>(jf, p.ds);
+    if constexpr (MM) {
+      const uint32_t jw = t.b0 + L::kMM64 + 4 * (j - t.b0);
+      const ulonglong2 q = sm_ld2_64<0>(jw);
+      sm_raise64<0>(jw, ~(uint64_t)p.mn, q.x);
+      sm_raise64<8>(jw, (uint64_t)p.mx, q.y);
+    }
+  }
+}
+
 // The window of rows [0, n) of vals, from 32 of them (called by one whole warp).
 template <int DT>
 __device__ __forceinline__ void s_window(const typename GV<DT>::T* vals, int64_t n, Window* w) {
@@ -1003,14 +1062,25 @@ __device__ __forceinline__ void s_window(const typename GV<DT>::T* vals, int64_t
     }
     if (lane == 0) w->base = b;
   } else if constexpr (is_float(DT)) {
-    uint32_t e = 0;
     constexpr uint32_t kInf = is_f32(DT) ? 0xFFu : 0x7FFu;
-    if (n > 0) {
-      if constexpr (is_f32(DT)) e = (__float_as_uint(vals[r]) >> 23) & 0xFFu;
-      else e = (uint32_t)((uint64_t)__double_as_longlong(vals[r]) >> 52) & 0x7FFu;
-      if (e == kInf) e = 0;
+    auto exponent = [&](int64_t i) -> uint32_t {
+      uint32_t e;
+      if constexpr (is_f32(DT)) e = (__float_as_uint(vals[i]) >> 23) & 0xFFu;
+      else e = (uint32_t)((uint64_t)__double_as_longlong(vals[i]) >> 52) & 0x7FFu;
+      return e == kInf ? 0u : e;
+    };
+    uint32_t e = __reduce_max_sync(0xffffffffu, n > 0 ? exponent(r) : 0u);
+    if (e == 0u && n > 32) {  // zeros only: a column of few other values shows one among 512 rows more
+      constexpr int kMore = 16;
+      const int64_t step = max(n / (32 * kMore), (int64_t)1);
+      uint32_t x[kMore];
+#pragma unroll
+      for (int u = 0; u < kMore; ++u) x[u] = exponent(min((lane * kMore + u) * step + step / 2, n - 1));
+#pragma unroll
+      for (int u = 0; u < kMore; ++u) e = max(e, x[u]);
+      e = __reduce_max_sync(0xffffffffu, e);
     }
-    const int top = (int)__reduce_max_sync(0xffffffffu, e) + 3;
+    const int top = (int)e + 3;
     if (lane == 0) w->ebase = max(1, min(top, (int)kInf - 1) - (is_f32(DT) ? 23 : 26));
   }
 }
@@ -1187,32 +1257,49 @@ __device__ __forceinline__ uint32_t build_rows(const BuildArgs& a, const STab<DT
         if constexpr (MULTI) {
           // Frequent keys among the warp's 128 rows go through one reduced
           // update each: first the key of lane 0's first row; while a key had
-          // at least kDominantRows rows, the next candidate is the first row not
-          // yet folded. The remaining rows take the per-row path.
-          uint32_t rem = has ? 0xFu : 0u;  // this lane's rows not yet folded
+          // at least kDominantRows rows, the next candidate is the first row of a
+          // key not yet looked at. The remaining rows take the per-row path.
+          uint32_t rem = has ? 0xFu : 0u;  // this lane's rows not yet folded, of keys not looked at
+          uint32_t late = 0u;              // of them, those of a key looked at
           uint32_t k0 = __shfl_sync(0xffffffffu, key[0], 0);
 #pragma unroll 1
           for (int w = 0; w < kMaxWarpKeys; ++w) {
             uint32_t take = 0;
 #pragma unroll
             for (int r = 0; r < 4; ++r) take |= (((rem >> r) & 1u) && key[r] == k0) ? (1u << r) : 0u;
-            if (__reduce_add_sync(0xffffffffu, (unsigned)__popc(take)) < (unsigned)kDominantRows) break;
-            if constexpr (SMEM && is_float(DT)) {  // rows outside the window take the per-row path
+            const uint32_t n = __reduce_add_sync(0xffffffffu, (unsigned)__popc(take));
+            if constexpr (SMEM && is_float(DT)) {
+              // few rows outside the window (and not zero) take the per-row path; more
+              // of them, and the key's rows are all summed as floats
+              if (n < (uint32_t)kDominantOther) break;
+              uint32_t in = take;
 #pragma unroll
-              for (int r = 0; r < 4; ++r) take &= s_enc<DT>(t, val[r]).ok ? 0xFu : ~(1u << r);
+              for (int r = 0; r < 4; ++r) in &= s_enc<DT>(t, val[r]).ok || val[r] == T(0) ? 0xFu : ~(1u << r);
+              if (__popc(__ballot_sync(0xffffffffu, take != in)) >= kDominantOther) {  // that many lanes
+                s_fold_warp_other<DT, MM>(a, t, k0, val, take);
+                rem &= ~take;
+              } else {
+                if (n < (uint32_t)kDominantRows) break;
+                s_fold_warp_key<DT, MM>(a, t, k0, val, in);
+                rem &= ~take;
+                late |= take & ~in;
+              }
+            } else {
+              if (n < (uint32_t)kDominantRows) break;
+              if constexpr (SMEM) s_fold_warp_key<DT, MM>(a, t, k0, val, take);
+              else g_fold_warp_key<DT, MM>(a, k0, val, take);
+              rem &= ~take;
             }
-            if constexpr (SMEM) s_fold_warp_key<DT, MM>(a, t, k0, val, take);
-            else g_fold_warp_key<DT, MM>(a, k0, val, take);
-            rem &= ~take;
             if (w + 1 == kMaxWarpKeys) break;
             const uint32_t lanes = __ballot_sync(0xffffffffu, rem != 0u);
             if (lanes == 0u) break;
-            uint32_t next = key[3];  // this lane's first row not yet folded
+            uint32_t next = key[3];  // this lane's first row of a key not yet looked at
             if (rem & 4u) next = key[2];
             if (rem & 2u) next = key[1];
             if (rem & 1u) next = key[0];
             k0 = __shfl_sync(0xffffffffu, next, __ffs(lanes) - 1);
           }
+          rem |= late;
           if (rem != 0u) {
             if constexpr (SMEM) s_fold<DT, MM, 4, false>(a, t, key, val, rem);
             else fold4_global(key, val, rem);
@@ -1254,7 +1341,8 @@ __device__ __forceinline__ uint32_t build_rows(const BuildArgs& a, const STab<DT
   }
 }
 
-// The build kernel of one query: grid-stride over all rows.
+// The build kernel of one query: grid-stride over all rows. 64 registers; one quad
+// a turn spills nothing but 48 bytes for float64 MIN/MAX with frequent keys.
 template <int DT, bool MM, bool SMEM, bool VEC, bool MULTI, int QPI = 1>
 __global__ void __launch_bounds__(1024, 1) gb_build(BuildArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
