@@ -192,7 +192,7 @@ typedef enum {
 /* Tuning knobs of agg_groupby; a zeroed struct (or NULL) selects defaults. */
 typedef struct agg_options {
   int32_t strategy;        /* agg_strategy */
-  int32_t block_threads;   /* threads per block of the build kernel; 0 = default */
+  int32_t block_threads;   /* threads per block of the build kernel (a partitioned SMEM build uses at most 512); 0 = default */
   int32_t blocks_per_sm;   /* resident blocks per SM; 0 = occupancy limit */
   int32_t smem_slots;      /* shared-memory table slots (power of two, <= 8192; a build uses at most 4096, 2048 for
                               partitioned MIN/MAX builds and float64 MIN/MAX); 0 = from the sketch */

@@ -439,7 +439,7 @@ class HashRun {
           return AGG_ERR_CUDA;
         }
         const size_t smem = stab_bytes_dt(vdt_, mm_, false);
-        const int threads = plan_.threads;
+        const int threads = std::min(plan_.threads, kTileThreads);
         KernelPtr bk = pick_tiles(vdt_, mm_, plan_.qpi);
         int bps = occupancy(bk, threads, smem);
         if (plan_.blocks_per_sm > 0 && plan_.blocks_per_sm < bps) bps = plan_.blocks_per_sm;
@@ -505,13 +505,14 @@ class HashRun {
     AGG_CUDA_TRY(cudaMemsetAsync(next_tile, 0, 8, s_));
     KernelPtr bk = pick_tiles(vdt_, mm_, plan_.qpi);
     const size_t smem = stab_bytes_dt(vdt_, mm_, false);
-    int bps = occupancy(bk, plan_.threads, smem);
+    const int threads = std::min(plan_.threads, kTileThreads);
+    int bps = occupancy(bk, threads, smem);
     if (plan_.blocks_per_sm > 0 && plan_.blocks_per_sm < bps) bps = plan_.blocks_per_sm;
     const int64_t grid = (int64_t)device_info().sm_count * bps;
     const longlong2* tl = tiles;
     const unsigned long long* nt = ntiles;
     void* args[] = {&a, &next_tile, &tile_rows, &tl, &nt};
-    cudaError_t e = cudaLaunchKernel(bk, dim3((unsigned)grid), dim3(plan_.threads), args, smem, s_);
+    cudaError_t e = cudaLaunchKernel(bk, dim3((unsigned)grid), dim3(threads), args, smem, s_);
     note_launch();
     if (e != cudaSuccess) {
       set_error("piecewise build launch failed: %s", cudaGetErrorString(e));

@@ -1378,9 +1378,10 @@ __global__ void __launch_bounds__(1024, 1) gb_build(BuildArgs a) {
 constexpr int64_t kPartTileRows = int64_t(1) << 16;
 // A tile never needs its cnt words settled.
 constexpr int64_t kTileRowsMax = kEpochRows;
+constexpr int kTileThreads = 512;  // at most: two blocks a SM of 64 registers a thread
 
 template <int DT, bool MM, bool VEC, int QPI = 1>
-__global__ void __launch_bounds__(512, 2) gb_build_tiles(BuildArgs a, unsigned long long* next_tile,
+__global__ void __launch_bounds__(kTileThreads, 2) gb_build_tiles(BuildArgs a, unsigned long long* next_tile,
                                                         int64_t tile_rows, const longlong2* tiles,
                                                         const unsigned long long* ntiles) {
   using T = typename GV<DT>::T;

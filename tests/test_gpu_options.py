@@ -1,0 +1,40 @@
+"""Build options and planned sizes of GROUP BY: block sizes on every build, table sizes of host-fed
+columns, the autotuner's choice as it is run, work items of a tuned batch."""
+import numpy as np
+import pytest
+import torch
+
+import datagen as dg
+import paper_2606_10030_gb300 as agg
+from tests.test_gpu_groupby import check_groups, run
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _build():
+    agg.build()
+    agg.lib()
+
+
+@pytest.mark.parametrize("dt", ["i32", "f64"])
+@pytest.mark.parametrize("threads", [64, 512, 544, 1024])
+@pytest.mark.parametrize("partition", [-1, 0, 1, 2])
+def test_every_block_size_on_every_build(partition, threads, dt):
+    """2^20 rows over 20 K keys: partition = 0 partitions them by itself."""
+    n = 1 << 20
+    k, v = dg.keys_uniform(n, 20_000, 1), dg.values(dt, n, 1)
+    res, _ = run(k, v, agg.AGG_STRAT_SMEM, partition=partition, block_threads=threads)
+    check_groups(res, k, v)
+
+
+@pytest.mark.parametrize("threads", [512, 1024])
+def test_every_block_size_on_host_fed_columns(threads):
+    """More than one chunk of 8 Mi rows, hash-partitioned chunk by chunk."""
+    n = (1 << 23) + 70_001
+    k, v = dg.keys_uniform(n, 200_000, 1), dg.values("i64", n, 1)
+    for partition in (-1, 1):
+        g = agg.agg_groupby_host(torch.from_numpy(k), torch.from_numpy(v), agg.AGG_ALL,
+                                 agg.options(agg.AGG_STRAT_SMEM, partition=partition, block_threads=threads))
+        check_groups(g.to_host(), k, v)
+        g.free()
