@@ -353,14 +353,7 @@ class HashRun {
     a.status = status_;
     a.progress = progress_;
     const bool tiled = plan_.partition && n >= kPartTileRows;
-    if (use_smem) {
-      // the unpartitioned build has the SM's shared memory to itself: its table
-      // is loaded to a quarter at most where the plan sized it for a half
-      const int most = stab_max_slots(vdt_, mm_, !tiled);
-      if (!tiled && !plan_.smem_given) plan_.smem_slots *= 2;
-      plan_.smem_slots = std::min(plan_.smem_slots, most);
-    }
-    a.smem_slots = use_smem ? plan_.smem_slots : 0;
+    a.smem_slots = use_smem ? shared_slots(tiled) : 0;
     if (tiled) return build_partitioned(a, use_smem);
     const int qpi = plan_.qpi ? plan_.qpi : 1;
     KernelPtr bk = pick_build(vdt_, mm_, use_smem, vec, plan_.multi_keys, qpi);
@@ -493,8 +486,7 @@ class HashRun {
     a.table = mem_;
     a.mask = (uint32_t)(plan_.slots - 1);
     a.gshift = 32 - (63 - __builtin_clzll((unsigned long long)plan_.slots));
-    plan_.smem_slots = std::min(plan_.smem_slots, stab_max_slots(vdt_, mm_, false));
-    a.smem_slots = plan_.smem_slots;
+    a.smem_slots = shared_slots(true);
     a.status = status_;
     a.progress = progress_;
     int64_t tile_rows = std::min(plan_.tile_rows ? (int64_t)plan_.tile_rows : kPartTileRows / 2, kTileRowsMax);
@@ -618,13 +610,21 @@ class HashRun {
     }
     g->num_groups = d;
     g->table_slots = plan_.slots;
-    g->smem_slots = plan_.strategy == AGG_STRAT_SMEM ? plan_.smem_slots : 0;
+    g->smem_slots = plan_.strategy == AGG_STRAT_SMEM ? used_slots_ ? used_slots_ : plan_.smem_slots : 0;
     g->strategy = plan_.strategy;
     *gout = g;
     return AGG_OK;
   }
 
  private:
+  // Slots of the shared tables of a build (the same for every build of a run).
+  // The unpartitioned build has the SM's shared memory to itself: its table is
+  // loaded to a quarter at most where the plan sized it for a half.
+  int shared_slots(bool tiled) {
+    const int slots = !tiled && !plan_.smem_given ? 2 * plan_.smem_slots : plan_.smem_slots;
+    return used_slots_ = std::min(slots, stab_max_slots(vdt_, mm_, !tiled));
+  }
+
   // One copy of the status block: status (+0), group count (+64), and the rows
   // seen / failed of a build stopped by a full table (+192, +200). Waits for
   // the stream; TABLE_FULL if the table overflowed.
@@ -656,6 +656,7 @@ class HashRun {
   void* mem_ = nullptr;
   int64_t nslots_ = 0;
   bool small_ = true, ranked_ = false;
+  int used_slots_ = 0;  // of the shared tables of the last build
   size_t status_off_ = 0, aux_off_ = 0;
   int* status_ = nullptr;
   unsigned long long* progress_ = nullptr;

@@ -38,3 +38,17 @@ def test_every_block_size_on_host_fed_columns(threads):
                                  agg.options(agg.AGG_STRAT_SMEM, partition=partition, block_threads=threads))
         check_groups(g.to_host(), k, v)
         g.free()
+
+
+def test_host_fed_column_keeps_its_planned_table():
+    """Three chunks of 8 Mi rows run on the table that the whole column on the device runs on."""
+    n = (1 << 24) + 1001
+    k, v = dg.keys_uniform(n, 100, 2), dg.values("i32", n, 2)
+    g = agg.agg_groupby(torch.from_numpy(k).cuda(), torch.from_numpy(v).cuda(), agg.AGG_ALL,
+                        agg.options(agg.AGG_STRAT_SMEM))
+    h = agg.agg_groupby_host(torch.from_numpy(k), torch.from_numpy(v), agg.AGG_ALL,
+                             agg.options(agg.AGG_STRAT_SMEM))
+    assert h.smem_slots == g.smem_slots == 512
+    check_groups(h.to_host(), k, v)
+    g.free()
+    h.free()
