@@ -476,13 +476,13 @@ agg_status agg_batch_tune(agg_batch_plan* plan, int reps, int32_t* tile_rows_out
  * parameters of GPU hash group-by, Sec. 7). Its axes: strategy, threads per
  * block, shared table size, rows a thread folds per iteration (4 or 8) and the
  * tile of a hash-partitioned build (16 Ki rows or the column-sized default).
- * Candidates: SMEM (sketch-sized table at 512 threads with 4 rows, with 8 rows,
- * with 16 Ki-row tiles, at 256 threads, and the largest table), GLOBAL at 256
+ * Candidates: SMEM (the build of an untuned call, and that with the largest
+ * table, at 256 threads, with 8 rows and with 16 Ki-row tiles), GLOBAL at 256
  * threads (4 rows) and 512 (8 rows), and SORT. Each is run on the actual query
  * and timed with CUDA events; the fastest is cached by query signature (value
  * dtype, ops, round(log2 n), rounded log2 of the distinct estimate, top-8
- * share decile, sortedness half). AGG_STRAT_AUTOTUNE uses the cache and tunes
- * on a miss; a batch's AGG_STRAT_AUTOTUNE queries take their strategy from the
+ * share decile, sortedness half). AGG_STRAT_AUTOTUNE runs with the options that
+ * the cached candidate was timed with, and tunes on a miss; a batch's AGG_STRAT_AUTOTUNE queries take their strategy from the
  * cache (the rule on a miss).
  */
 #define AGG_TUNE_MAX 8
@@ -490,8 +490,8 @@ typedef struct agg_tune_result {
   int32_t ncand;                    /* candidates timed */
   int32_t best;                     /* index of the fastest */
   int32_t strategy[AGG_TUNE_MAX];   /* AGG_STRAT_SMEM / GLOBAL / SORT */
-  int32_t threads[AGG_TUNE_MAX];
-  int32_t smem_slots[AGG_TUNE_MAX];
+  int32_t threads[AGG_TUNE_MAX];    /* 0: the build's own choice */
+  int32_t smem_slots[AGG_TUNE_MAX]; /* of the shared tables it ran on */
   int32_t items_per_thread[AGG_TUNE_MAX];
   int32_t tile_rows[AGG_TUNE_MAX];  /* 0: the column-sized default */
   float ms[AGG_TUNE_MAX];           /* device time of the whole agg_groupby call */

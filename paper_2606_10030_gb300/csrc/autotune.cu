@@ -15,8 +15,8 @@ namespace agg {
 
 struct TuneChoice {
   int strategy;
-  int threads;
-  int smem_slots;
+  int threads;     // 0: the build's own choice
+  int smem_slots;  // 0: planned from the sketch
   int items;  // rows a thread folds per iteration (4 or 8)
   int tile;   // rows per tile of a hash-partitioned build (0: from the column)
 };
@@ -38,32 +38,23 @@ agg_status groupby_with(const uint32_t* keys, const void* vals, int64_t n, int v
                         const agg_options& o, cudaStream_t s, agg_groups** out, const float* known_feat,
                         double known_hll);
 
-static int smem_slots_sized(const float* f, bool mm) {
-  bool covered = false;
-  const double est = distinct_estimate(f, &covered);
-  const int maxs = mm ? 2048 : 4096;
-  int64_t sl = next_pow2((int64_t)std::ceil(2.0 * est));
-  if (sl < 256) sl = 256;
-  if (sl > maxs) sl = maxs;
-  return (int)sl;
-}
-
 static agg_status run_candidates(const uint32_t* keys, const void* vals, int64_t n, int vdt, uint32_t ops,
                                  const float* feat, double hll, int reps, cudaStream_t s, agg_tune_result* r) {
   std::memset(r, 0, sizeof(*r));
   std::memcpy(r->features, feat, sizeof(float) * F_COUNT);
-  const bool mm = ops_minmax(ops);
-  const int sized = smem_slots_sized(feat, mm), maxs = mm ? 2048 : 4096;
+  const int most = vdt == AGG_F64 && ops_minmax(ops) ? 2048 : 4096;  // slots of the largest shared table
   // axes: strategy; block size; shared table size; rows a thread folds per
   // iteration (4 or 8); tile of the hash-partitioned build (16 Ki rows or the
-  // column-sized default; the build runs on tiles only when it partitions)
+  // column-sized default; the build runs on tiles only when it partitions).
+  // The first candidate is an untuned call's shared-memory build, and the
+  // others change one axis of it.
   TuneChoice c[AGG_TUNE_MAX];
   int nc = 0;
-  c[nc++] = {AGG_STRAT_SMEM, 512, sized, 4, 0};
-  if (maxs != sized) c[nc++] = {AGG_STRAT_SMEM, 512, maxs, 4, 0};
-  c[nc++] = {AGG_STRAT_SMEM, 256, sized, 4, 0};
-  c[nc++] = {AGG_STRAT_SMEM, 512, sized, 8, 0};
-  c[nc++] = {AGG_STRAT_SMEM, 512, sized, 4, 16384};
+  c[nc++] = {AGG_STRAT_SMEM, 0, 0, 4, 0};
+  c[nc++] = {AGG_STRAT_SMEM, 0, most, 4, 0};
+  c[nc++] = {AGG_STRAT_SMEM, 256, 0, 4, 0};
+  c[nc++] = {AGG_STRAT_SMEM, 0, 0, 8, 0};
+  c[nc++] = {AGG_STRAT_SMEM, 0, 0, 4, 16384};
   c[nc++] = {AGG_STRAT_GLOBAL, 256, 0, 4, 0};
   c[nc++] = {AGG_STRAT_GLOBAL, 512, 0, 8, 0};
   c[nc++] = {AGG_STRAT_SORT, 0, 0, 0, 0};
@@ -93,12 +84,12 @@ static agg_status run_candidates(const uint32_t* keys, const void* vals, int64_t
       cudaEventSynchronize(b);
       float ms = 0.f;
       cudaEventElapsedTime(&ms, a, b);
+      r->smem_slots[i] = g->smem_slots;
       agg_groups_free(g);
       best = std::min(best, ms);
     }
     r->strategy[i] = c[i].strategy;
     r->threads[i] = c[i].threads;
-    r->smem_slots[i] = c[i].smem_slots;
     r->items_per_thread[i] = c[i].items;
     r->tile_rows[i] = c[i].tile;
     r->ms[i] = best;
@@ -117,37 +108,37 @@ static agg_status run_candidates(const uint32_t* keys, const void* vals, int64_t
   return AGG_OK;
 }
 
-bool autotune_cached(int vdt, uint32_t ops, const float* feat, int* strategy, int* smem_slots) {
+static bool cached(int vdt, uint32_t ops, const float* feat, TuneChoice* c) {
   std::lock_guard<std::mutex> lk(g_tmu);
   auto it = g_cache.find(signature(vdt, ops, feat));
   if (it == g_cache.end()) return false;
-  *strategy = it->second.strategy;
-  *smem_slots = it->second.smem_slots;
+  *c = it->second;
   return true;
 }
 
+bool autotune_cached(int vdt, uint32_t ops, const float* feat, int* strategy) {
+  TuneChoice c;
+  if (!cached(vdt, ops, feat, &c)) return false;
+  *strategy = c.strategy;
+  return true;
+}
+
+// The options that the fastest candidate was timed with, in place of o's.
 agg_status autotune_pick(const uint32_t* keys, const void* vals, int64_t n, int vdt, uint32_t ops,
-                         const float* feat, double hll, cudaStream_t s, int* strategy, int* smem_slots,
-                         int64_t* table_slots, int* items, int* tile_rows) {
-  *table_slots = 0;
-  {
-    std::lock_guard<std::mutex> lk(g_tmu);
-    auto it = g_cache.find(signature(vdt, ops, feat));
-    if (it != g_cache.end()) {
-      *strategy = it->second.strategy;
-      *smem_slots = it->second.smem_slots;
-      *items = it->second.items;
-      *tile_rows = it->second.tile;
-      return AGG_OK;
-    }
+                         const float* feat, double hll, cudaStream_t s, agg_options* o) {
+  TuneChoice c;
+  if (!cached(vdt, ops, feat, &c)) {
+    agg_tune_result r;
+    agg_status st = run_candidates(keys, vals, n, vdt, ops, feat, hll, 1, s, &r);
+    if (st != AGG_OK) return st;
+    if (!cached(vdt, ops, feat, &c)) c = {r.strategy[r.best], 0, 0, 0, 0};  // cleared meanwhile
   }
-  agg_tune_result r;
-  agg_status st = run_candidates(keys, vals, n, vdt, ops, feat, hll, 1, s, &r);
-  if (st != AGG_OK) return st;
-  *strategy = r.strategy[r.best];
-  *smem_slots = r.smem_slots[r.best];
-  *items = r.items_per_thread[r.best];
-  *tile_rows = r.tile_rows[r.best];
+  o->strategy = c.strategy;
+  if (o->block_threads == 0) o->block_threads = c.threads;
+  if (c.smem_slots != 0) o->smem_slots = c.smem_slots;
+  o->table_slots = 0;
+  o->items_per_thread = c.items;
+  o->tile_rows = c.tile;
   return AGG_OK;
 }
 
@@ -220,6 +211,8 @@ extern "C" agg_status agg_autotune_load(const char* path) {
                     &v[8], &v[9], &v[10]) != 11)
       continue;
     if (v[6] < AGG_STRAT_SMEM || v[6] > AGG_STRAT_SORT) continue;
+    if (v[7] != 0 && (v[7] < 64 || v[7] > 1024 || v[7] % 32 != 0)) continue;
+    if (v[8] != 0 && (v[8] < 64 || v[8] > 8192 || (v[8] & (v[8] - 1)) != 0)) continue;
     if (v[9] != 0 && v[9] != 4 && v[9] != 8) continue;
     if (v[10] != 0 && (v[10] < 4096 || v[10] > 65536 || (v[10] & (v[10] - 1)) != 0)) continue;
     g_cache[Sig(v[0], v[1], v[2], v[3], v[4], v[5])] = TuneChoice{v[6], v[7], v[8], v[9], v[10]};

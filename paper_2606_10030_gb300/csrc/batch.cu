@@ -589,8 +589,8 @@ static void plan_sizes(agg_batch_plan* P, const std::vector<int>& learned) {
     int strat = q.strategy;
     if (strat == AGG_STRAT_LEARNED) strat = learned[i] >= 0 ? learned[i] : rule_strategy(f, q.ops);
     else if (strat == AGG_STRAT_AUTOTUNE) {
-      int sslots = 0;  // the autotuner's cached choice for this signature, else the rule
-      if (!autotune_cached(q.dtype, q.ops, f, &strat, &sslots)) strat = rule_strategy(f, q.ops);
+      // the autotuner's cached choice for this signature, else the rule
+      if (!autotune_cached(q.dtype, q.ops, f, &strat)) strat = rule_strategy(f, q.ops);
     } else if (strat == AGG_STRAT_AUTO) {
       strat = rule_strategy(f, q.ops);
     }

@@ -681,8 +681,7 @@ int select_learned(const float* feat, bool* ok);
 agg_status sketch_and_select(const uint32_t* keys, int64_t n, int vdt, uint32_t ops, uint64_t offset,
                              cudaStream_t s, float* feat, int* strategy);
 agg_status autotune_pick(const uint32_t* keys, const void* vals, int64_t n, int vdt, uint32_t ops,
-                         const float* feat, double hll, cudaStream_t s, int* strategy, int* smem_slots,
-                         int64_t* table_slots, int* items, int* tile_rows);
+                         const float* feat, double hll, cudaStream_t s, agg_options* o);
 
 // Sketch the keys on the device and read the features back (one sync).
 agg_status sketch_features(const uint32_t* keys, int64_t n, int vdt, uint32_t ops, uint64_t offset,
@@ -762,32 +761,30 @@ int64_t table_slots_for(const float* feat, int64_t n, double hll) {
 }
 
 static agg_status choose(const uint32_t* keys, const void* vals, int64_t n, int vdt, uint32_t ops,
-                         const agg_options& o, const float* feat, bool have_feat, double hll, cudaStream_t s,
+                         const agg_options& opts, const float* feat, bool have_feat, double hll, cudaStream_t s,
                          Choice* c) {
+  agg_options o = opts;
   bool covered = false;
   double est = have_feat ? distinct_estimate(feat, &covered) : 1024.0;
   if (hll > 0.0) est = hll;
+  if (o.strategy == AGG_STRAT_AUTOTUNE) {
+    agg_status st = autotune_pick(keys, vals, n, vdt, ops, feat, hll, s, &o);
+    if (st != AGG_OK) return st;
+  }
   int strategy = o.strategy;
-  int64_t tslots = o.table_slots;
-  int sslots = o.smem_slots;
-  int items = o.items_per_thread;
-  int tile = o.tile_rows;
   if (strategy == AGG_STRAT_LEARNED) {
     bool ok = false;
     strategy = select_learned(feat, &ok);
     if (!ok) strategy = rule_strategy(feat, ops, hll);
-  } else if (strategy == AGG_STRAT_AUTOTUNE) {
-    agg_status st = autotune_pick(keys, vals, n, vdt, ops, feat, hll, s, &strategy, &sslots, &tslots, &items, &tile);
-    if (st != AGG_OK) return st;
   } else if (strategy == AGG_STRAT_AUTO) {
     strategy = have_feat ? rule_strategy(feat, ops, hll) : AGG_STRAT_GLOBAL;
   }
   c->strategy = strategy;
   c->plan.strategy = strategy;
-  c->plan.slots = tslots ? tslots
+  c->plan.slots = o.table_slots ? o.table_slots
                          : hll > 0.0 ? slots_for_count(hll, n) : (have_feat ? table_slots_from_sketch(feat, n) : 2048);
-  c->plan.smem_slots = sslots ? std::min(sslots, stab_max_slots(vdt, ops_minmax(ops), true))
-                              : smem_slots_for(est, stab_max_slots(vdt, ops_minmax(ops), true));
+  c->plan.smem_slots = o.smem_slots ? std::min(o.smem_slots, stab_max_slots(vdt, ops_minmax(ops), true))
+                                    : smem_slots_for(est, stab_max_slots(vdt, ops_minmax(ops), true));
   c->plan.threads_given = o.block_threads != 0;
   c->plan.smem_given = o.smem_slots != 0;
   c->plan.threads = o.block_threads ? o.block_threads : (strategy == AGG_STRAT_SMEM ? 512 : 256);
@@ -795,8 +792,8 @@ static agg_status choose(const uint32_t* keys, const void* vals, int64_t n, int 
   // the warp-level reduction of several keys pay; without a sketch, assume so
   c->plan.multi_keys = !have_feat || feat[F_TOP1] >= 0.03f || est <= 32.0;
   c->plan.blocks_per_sm = o.blocks_per_sm;
-  c->plan.qpi = items == 8 ? 2 : items == 4 ? 1 : 0;
-  c->plan.tile_rows = tile;
+  c->plan.qpi = o.items_per_thread == 8 ? 2 : o.items_per_thread == 4 ? 1 : 0;
+  c->plan.tile_rows = o.tile_rows;
   // Partition the rows by hash first when the shared tables would spill (more
   // distinct keys than a shared table admits) or the global table exceeds
   // half of L2; each partition then has about 1/256 of the keys.

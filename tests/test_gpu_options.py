@@ -52,3 +52,23 @@ def test_host_fed_column_keeps_its_planned_table():
     check_groups(h.to_host(), k, v)
     g.free()
     h.free()
+
+
+@pytest.mark.parametrize("keys", [100, 1000, 3000])
+@pytest.mark.parametrize("dt", ["i32", "i64", "f64"])
+def test_autotuned_call_runs_the_timed_build(dt, keys):
+    """AUTOTUNE's table is the one timed; the shared-memory default among the candidates is AUTO's own."""
+    agg.lib().agg_autotune_clear()
+    n = 1 << 21
+    k = torch.from_numpy(dg.keys_uniform(n, keys, 3)).cuda()
+    v = torch.from_numpy(dg.values(dt, n, 3)).cuda()
+    r = agg.agg_autotune(k, v, agg.AGG_ALL, reps=2)
+    auto = agg.agg_groupby(k, v, agg.AGG_ALL, agg.options(agg.AGG_STRAT_SMEM))
+    smem = [s for s, t in zip(r.smem_slots, list(r.strategy)[:r.ncand]) if t == agg.AGG_STRAT_SMEM]
+    assert auto.smem_slots in smem
+    g = agg.agg_groupby(k, v, agg.AGG_ALL, agg.options(agg.AGG_STRAT_AUTOTUNE))
+    assert g.strategy == r.strategy[r.best]
+    if g.strategy == agg.AGG_STRAT_SMEM:
+        assert g.smem_slots == r.smem_slots[r.best]
+    auto.free()
+    g.free()
