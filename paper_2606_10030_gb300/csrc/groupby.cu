@@ -726,15 +726,21 @@ bool wants_hll(const float* f, int64_t n) {
   return n >= (int64_t(1) << 22) && 1.0 - (double)f[F_F1] < 0.97;
 }
 
-// A column that the rule sorts whatever its HyperLogLog count, which then is
-// not taken: so few repeats in the sample that it has more than about n^2 / 2.4e8
-// keys. (A sample of m rows repeats C(m, 2) sum p^2 >= m^2 / 2d times, so
-// frequent keys cannot hide.) Sorted without the count against partitioned with
-// it, float64: 4.2 M rows of 65 K keys 0.35 ms against 0.37; 9 M rows of 140 K
-// 0.55 against 0.47, of 560 K 0.56 against 0.61; 16 M rows of 250 K 0.86
-// against 0.64, of 1 M 0.88 against 0.89. From 2^25 rows on the sample no
-// longer tells such counts.
-bool sorts_uncounted(const float* f, int64_t n) {
+// A column whose HyperLogLog count does not pay for itself under AUTO, which then
+// chooses from the sample alone: so few repeats in the sample that it has more than
+// about n^2 / 2.4e8 keys, under 2^25 rows. (A sample of m rows repeats C(m, 2)
+// sum p^2 >= m^2 / 2d times, so frequent keys cannot hide.) Nearly all of these
+// are sorted, where the count would have partitioned those of 12 or 16 rows a key
+// and more; and flat ones of fewer than 10^5 keys (up to 4.9 M rows) are built on
+// partitioned shared tables of the sample's size. Uncounted against partitioned
+// with the count, int32 SUM/COUNT/MIN/MAX and float64 SUM/COUNT: 4.3 M rows of 85 K
+// keys 256 us against 299 and 306 against 351 (sorted 289 and 305), of 120 K keys
+// 287 against 316 and 302 against 375 (both sorted); 6 M rows of 150 K keys 348
+// against 319 and 369 against 362, of 300 K 346 against 370 and 366 against 396; 9 M
+// of 330 K 441 against 434 and 469 against 471; 16 M of 1.05 M level; 24 M of 2.4 M
+// 947 against 1316 and 1018 against 1119. From 2^25 rows on the sample no longer
+// tells such counts.
+bool planned_uncounted(const float* f, int64_t n) {
   if (n >= (int64_t(1) << 25)) return false;
   const double repeats = (1.0 - (double)f[F_DISTINCT]) * (double)kSketchSample;
   return repeats * (double)n * (double)n <= 2e15;
@@ -913,7 +919,7 @@ agg_status groupby_with(const uint32_t* keys, const void* vals, int64_t n, int v
     st = sketch_features(keys, n, vdt, ops, o.sample_offset, s, feat);
     if (st != AGG_OK) return st;
     have = true;
-    if (wants_hll(feat, n) && !(o.strategy == AGG_STRAT_AUTO && sorts_uncounted(feat, n))) {
+    if (wants_hll(feat, n) && !(o.strategy == AGG_STRAT_AUTO && planned_uncounted(feat, n))) {
       st = hll_estimate(keys, n, s, &hll, part_counts);
       if (st != AGG_OK) return st;
       have_counts = true;
