@@ -585,7 +585,7 @@ def extra_batched(steps: int, nq: int = 512) -> dict:
         return wall, sum(v[0] for v in agg.profile_read().values()) / steps
 
     time_runs()  # warm-up replays (the first replays after a capture run slower)
-    fixed_s, fixed_gpu_ms = time_runs()  # the default 64 Ki-row work items
+    fixed_s, fixed_gpu_ms = time_runs()  # the plan's own work items
     tile = plan.tune(2)  # the autotuner's tile axis: 16, 32 or 64 Ki rows
     time_runs()  # warm-up replays of the re-planned graph
     batch_s, batch_gpu_ms = time_runs()

@@ -465,10 +465,12 @@ agg_status agg_batch_result(const agg_batch_plan* plan, int i, agg_groups** out)
 int agg_batch_size(const agg_batch_plan* plan);
 void agg_batch_plan_free(agg_batch_plan* plan);
 agg_status agg_batch(const agg_query* queries, int nq, agg_groups** outs, void* stream);
-/* The autotuner's tile axis for a batch: time `reps` runs of the plan at each
-   work-item size of 16, 32 and 64 Ki rows (each captured as its own graph),
-   keep the fastest and write it to *tile_rows_out (may be NULL). Results of
-   the runs are those of agg_batch_run. Synchronous. */
+/* The autotuner's tile axis for a batch: time `reps` runs of the plan at its
+   present work-item size and at 16, 32 and 64 Ki rows (65536 runs as 65532-row
+   items; each size captured as its own graph) and keep the fastest. The fastest
+   of the latter three is written to *tile_rows_out (may be NULL); a small
+   batch's own items may be smaller still, and faster. Results of the runs are
+   those of agg_batch_run. Synchronous. */
 agg_status agg_batch_tune(agg_batch_plan* plan, int reps, int32_t* tile_rows_out, void* stream);
 
 /*

@@ -667,7 +667,8 @@ class BatchPlan:
         check(lib().agg_batch_run(self._h, _stream_ptr(stream)))
 
     def tune(self, reps: int = 2, stream=None) -> int:
-        """Pick the fastest work-item size (16, 32 or 64 Ki rows) by timing runs; returns it."""
+        """Keep the fastest work-item size of the plan's own and 16, 32 and 64 Ki rows by timing runs;
+        returns the fastest of the latter three."""
         t = ctypes.c_int32(0)
         check(lib().agg_batch_tune(self._h, reps, ctypes.byref(t), _stream_ptr(stream)))
         return int(t.value)

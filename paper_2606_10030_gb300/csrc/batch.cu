@@ -792,9 +792,12 @@ extern "C" agg_status agg_batch_tune(agg_batch_plan* P, int reps, int32_t* tile_
   clear_error();
   AGG_CHECK_ARG(P != nullptr, "null plan");
   cudaStream_t s = (cudaStream_t)stream;
-  const int64_t cand[] = {16384, 32768, 65536};
-  float best_ms = INFINITY;
-  int64_t best = P->tile_rows;
+  // the plan's own size (8 Ki rows for a batch of few rows) is timed first and
+  // kept unless one of the axis is faster
+  const int64_t own = P->tile_rows;
+  const int64_t cand[] = {own, 16384, 32768, 65536};
+  float best_ms = INFINITY, axis_ms = INFINITY;
+  int64_t best = own, axis = 16384;
   cudaEvent_t a, b;
   AGG_CUDA_TRY(cudaEventCreate(&a));
   AGG_CUDA_TRY(cudaEventCreate(&b));
@@ -817,6 +820,10 @@ extern "C" agg_status agg_batch_tune(agg_batch_plan* P, int reps, int32_t* tile_
       best_ms = ms;
       best = t;
     }
+    if (t >= 16384 && ms < axis_ms) {
+      axis_ms = ms;
+      axis = t;
+    }
   }
   cudaEventDestroy(a);
   cudaEventDestroy(b);
@@ -825,7 +832,7 @@ extern "C" agg_status agg_batch_tune(agg_batch_plan* P, int reps, int32_t* tile_
     st = plan_retile(P, best, s);
     if (st != AGG_OK) return st;
   }
-  if (tile_rows_out) *tile_rows_out = (int32_t)best;
+  if (tile_rows_out) *tile_rows_out = (int32_t)axis;
   return AGG_OK;
 }
 

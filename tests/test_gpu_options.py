@@ -72,3 +72,34 @@ def test_autotuned_call_runs_the_timed_build(dt, keys):
         assert g.smem_slots == r.smem_slots[r.best]
     auto.free()
     g.free()
+
+
+def _ms(f, reps=20):
+    for _ in range(3):
+        f()
+    torch.cuda.synchronize()
+    out = []
+    for _ in range(5):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        for _ in range(reps):
+            f()
+        b.record()
+        torch.cuda.synchronize()
+        out.append(a.elapsed_time(b) / reps)
+    return min(out)
+
+
+def test_tuning_a_small_batch_does_not_slow_it_down():
+    """131 K float64 rows over 64 K keys: a work item is a chain of atomics, so that 16 Ki rows an item
+    take nearly twice the plan's own 8 Ki."""
+    n = 1 << 17
+    k, v = dg.keys_uniform(n, 1 << 16, 4), dg.values("f64", n, 4)
+    plan = agg.BatchPlan([(torch.from_numpy(k).cuda(), torch.from_numpy(v).cuda(), agg.AGG_ALL, agg.AGG_STRAT_AUTO)])
+    before = _ms(plan.run)
+    assert plan.tune(5) in (16384, 32768, 65536)
+    assert _ms(plan.run) <= 1.15 * before
+    g = plan.result(0)
+    check_groups(g.to_host(), k, v)
+    g.free()
+    plan.free()
