@@ -27,10 +27,13 @@
  *    zero-extended. It is exact and bit-identical for any reduction order.
  *  - Float SUM is returned in float64. Float32 columns are summed with
  *    TwoSum-compensated float32 partials whose final merge runs in float64.
- *    The ungrouped scan sums float64 columns per thread as 128-bit
- *    fixed-point integers (scaled to the largest exponent the thread has
- *    seen) and merges them as float64 pairs; GROUP BY adds float64 values in
- *    float64.
+ *    The ungrouped scan sums float64 columns per thread as fixed-point
+ *    integers (scaled to the largest exponent the thread has seen), and merges
+ *    the sums of both float types as 128-bit fixed-point integers with what
+ *    lies below their unit beside them in float64. GROUP BY's shared tables add
+ *    float rows as exact fixed point inside a window of exponents that the
+ *    block chooses from a sample; other rows, the global table and the sort
+ *    strategy add in float64 (float32: compensated float32 pairs first).
  *  - MIN/MAX of floats use the total order -0.0 < +0.0; inputs hold no NaN.
  *  - AVG = (double)SUM / (double)COUNT.
  */

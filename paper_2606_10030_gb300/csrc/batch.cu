@@ -57,7 +57,9 @@ struct BQ {  // one query of a batch, on the device
 };
 
 // Out of line, so that each type's tile gets the kernel's whole register budget
-// (inlined into one kernel, the forty variants spilled a kilobyte a thread).
+// (inlined into one kernel, the forty variants spilled a kilobyte a thread; as
+// functions they store 16 bytes, int32 sums, to 250, float64 MIN/MAX, the
+// registers saved for the caller included).
 template <int DT, bool MM, bool SMEM>
 __device__ __noinline__ void batch_tile(const BQ& q, int64_t r0, int64_t r1, unsigned char* smem) {
   BuildArgs a;

@@ -1342,7 +1342,8 @@ __device__ __forceinline__ uint32_t build_rows(const BuildArgs& a, const STab<DT
 }
 
 // The build kernel of one query: grid-stride over all rows. 64 registers; one quad
-// a turn spills nothing but 48 bytes for float64 MIN/MAX with frequent keys.
+// a turn spills nothing but 8 to 44 bytes for int64 and float64 MIN/MAX with
+// frequent keys, two quads (on request) up to 164.
 template <int DT, bool MM, bool SMEM, bool VEC, bool MULTI, int QPI = 1>
 __global__ void __launch_bounds__(1024, 1) gb_build(BuildArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -1374,7 +1375,9 @@ __global__ void __launch_bounds__(1024, 1) gb_build(BuildArgs a) {
 // table region they update stays in L2; each tile clears its shared table
 // first and merges it into the global table at the end. With a tile list
 // (rows partitioned chunk by chunk), tile t is the row range tiles[t] =
-// (first row, rows), *ntiles of them, listed partition by partition.
+// (first row, rows), *ntiles of them, listed partition by partition. 64 registers;
+// one quad a turn spills 24 to 68 bytes, 120 for float64 MIN/MAX, two quads (on
+// request) 36 to 252.
 constexpr int64_t kPartTileRows = int64_t(1) << 16;
 // A tile never needs its cnt words settled.
 constexpr int64_t kTileRowsMax = kEpochRows;
