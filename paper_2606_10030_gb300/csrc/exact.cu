@@ -112,13 +112,13 @@ __global__ void __launch_bounds__(kExactThreads) exact_add(const uint32_t* __res
 // keys (buckets of 4 slots, at most half full, with each key's group number)
 // and for every group W words of 32 bits, digits of 16 bits: a value adds at
 // most 65535 to each of 3 (float32) or 5 (float64) neighbouring digits, with
-// native shared atomics that return nothing. After kExactEpoch rows the block
+// native shared atomics that return nothing. After kExactIters iterations the block
 // carries the digits into their 16 bits; the last two digits hold the growth
 // of 2^32 rows. Few groups get several copies of their words, one per lane
 // class, so that a warp's rows of one group do not serialise. Against 64-bit
 // atomics in HBM after a binary search: 2^25 float32 rows over 4096 keys 2100
 // -> 153 us; bound by the shared-memory wavefronts of the lookup and the
-// three updates (about 35 a warp row).
+// three updates (30 a warp and 32 rows).
 constexpr int kExactSmemThreads = 1024;
 constexpr int kExactRows = 4;                                                  // rows a thread adds per iteration
 constexpr int kExactIters = 32767 / (kExactSmemThreads * kExactRows);          // iterations between two carries

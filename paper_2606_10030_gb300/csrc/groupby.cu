@@ -617,7 +617,8 @@ class HashRun {
   }
 
  private:
-  // Slots of the shared tables of a build (the same for every build of a run).
+  // Slots of the shared tables of a build, from the plan alone: the same for every
+  // build of a run that is tiled, and for every one that is not.
   // The unpartitioned build has the SM's shared memory to itself: its table is
   // loaded to a quarter at most where the plan sized it for a half.
   int shared_slots(bool tiled) {

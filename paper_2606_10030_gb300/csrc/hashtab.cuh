@@ -361,16 +361,17 @@ __device__ __forceinline__ void report_counts(const BuildArgs& a, const BlockCou
 // by the shared address of its key word, and every update is one instruction
 // with an immediate offset.
 //
-// What bounds it: warp instructions, then shared-memory wavefronts. The earlier
+// What bounds it: shared-memory wavefronts, then warp instructions. The earlier
 // fold (generic pointers, one row at a time, an out-of-line lookup for every
 // key outside its home bucket, predicated and branched updates, carries added
-// separately) took 175 warp instructions and 1.22 wavefronts a row on int64
+// separately) took 175 instructions and 39 wavefronts a warp and 32 rows on int64
 // SUM/COUNT/MIN/MAX over 1024 keys; four rows folded phase by phase (lookups,
-// sum updates, extremes) with unconditional updates take 87 and 1.1. Builds:
-// 2^26 int64 rows over 1024 keys 0.412 -> 0.284 ms; 2^28 float32 rows over 14 M
-// keys (partitioned) 3.41 -> 2.40 ms; 2^30 int64 rows over 2^16 keys
-// (partitioned) 6.51 -> 5.36 ms; 16 M float64 rows over 2^20 keys (partitioned)
-// 0.47 -> 0.33 ms. Every update is a native 32-bit shared atomic:
+// sum updates, extremes) with unconditional updates take 76 and 32 (L1 pipe 89 %
+// busy, issue 46 %). Builds: 2^26 int64 rows over 1024 keys 0.412 -> 0.284 ms;
+// 2^28 float32 rows over 14 M keys (partitioned) 3.41 -> 2.48 ms; 2^30 int64 rows
+// over 2^16 keys (partitioned) 6.51 -> 5.38 ms; 16 M float64 rows over 2^20 keys
+// (partitioned) 0.47 -> 0.33 ms. Every update but those of rows outside the window
+// is a native 32-bit shared atomic:
 //   count   low half of the cnt word; its high half counts, for integers, the
 //           carries out of the sum's low word (one atomic adds the row and its
 //           carry) and, for floats, the negative rows (below). A block folds at

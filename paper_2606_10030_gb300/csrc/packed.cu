@@ -18,7 +18,7 @@
 // HBM: 104 us a call when every value computed its own 64-bit position and was
 // folded as a whole value and a second launch merged, 40.6 us with the words
 // loaded where they are used, 30.9 us now (2.3 TB/s), bound by the instructions of
-// the extraction (19 a warp and 32 values) and the latency of its shared loads.
+// the extraction (22 a warp and 32 values, issue 72 %) and the latency of its shared loads.
 #include <algorithm>
 #include <cstring>
 #include <map>

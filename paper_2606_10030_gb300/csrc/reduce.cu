@@ -22,7 +22,7 @@
 // merge them with integer additions; one thread converts the total to float64 at
 // the end. The order is fixed, so the result is deterministic for a given grid.
 // Measured against float64 TwoSum merges in every shuffle step: 2^20 int32 rows
-// 17.7 -> 8.7 us a call, 10^8 float64 rows 207 -> 158 us (with the scale started
+// 17.7 -> 8.7 us a call, 10^8 float64 rows 207 -> 160 us (with the scale started
 // from the warp's first rows, two rows sharing the fast-path and MIN/MAX tests,
 // SUM alone 168 -> 127, and the extremes shared by the warp after each iteration:
 // a thread of 430 rows moves its own a dozen times, and each time its warp goes
